@@ -68,25 +68,52 @@ __device__ __forceinline__ float cvt<float, double>(double d) {
 }
 #endif
 
-// 1/d.  On the GPU in FP64: the FP32 hardware reciprocal of d as the seed
-// r0 (relative error e = 1 - d r0 below 2^-22 with the truncated
-// conversion), then one polynomial correction r0 (1 + e + e^2) of the
-// Newton-Raphson family for the reciprocal, whose relative error is O(e^3)
-// (below 1e-19): three FMAs.  Values outside the FP32 normal range use the
-// division.  Elsewhere (host, FP32, counting types): the plain division.
+// 1/d.  On the GPU without branches, so that the some 170 reciprocals of a
+// step attempt leave the straight-line code in one piece (the compiler can
+// schedule across them and share equal ones).
+//   FP64: the significand of d as a float in [1, 2), the hardware's
+//     approximate FP32 reciprocal of it widened and rescaled by integer
+//     operations into the seed r0 (relative error e = 1 - d r0 below 2^-21),
+//     then one polynomial correction r0 (1 + e + e^2) of the Newton-Raphson
+//     family for the reciprocal, whose relative error is O(e^3) (below
+//     1e-18): three FMAs on the FP64 pipe.  |d| below 2^-1022 gives a
+//     signed infinity, |d| from 2^1022 on a signed zero, NaN stays NaN.
+//   FP32: the approximate reciprocal and one Newton-Raphson step with the
+//     residual from an FMA (rounded to nearest but for near-ties); d = 0,
+//     infinite or NaN keeps the approximation, which is exact there.
+// Elsewhere (host, counting types): the plain division.
 template <class R>
 CHAD_HD R rcp(R d) {
   return R(1) / d;
 }
+__device__ __forceinline__ float rcp_approx(float d) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
+  return r;
+}
 #ifdef __CUDA_ARCH__
 template <>
+__device__ __forceinline__ float rcp<float>(float d) {
+  const float r = rcp_approx(d);
+  const float e = fmaf(-d, r, 1.0f);
+  const float x = fmaf(r, e, r);
+  return fabsf(e) < 0.5f ? x : r;
+}
+template <>
 __device__ __forceinline__ double rcp<double>(double d) {
-  const float f = cvt<float, double>(d);
-  const float af = fabsf(f);
-  if (!(af > 1e-30f && af < 1e30f)) return 1.0 / d;
-  const double r = cvt<double, float>(__frcp_rn(f));
+  const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+  const unsigned sgn = hi & 0x80000000u, mag = hi & 0x7fffffffu;
+  const float m = __uint_as_float(0x3f800000u | ((hi & 0xfffffu) << 3) | (lo >> 29));
+  const unsigned s = __float_as_uint(rcp_approx(m));  // in [1/2, 1]
+  // exponents: the seed's (bias 127 -> 1023) minus that of d
+  const unsigned rh = sgn | ((s >> 3) + 0x77f00000u - (mag & 0x7ff00000u));
+  const double r = __hiloint2double((int)rh, (int)(s << 29));
   const double e = fma(-d, r, 1.0);
-  return fma(r, fma(e, e, e), r);
+  const double x = fma(r, fma(e, e, e), r);
+  // on the bit patterns: tiny -> infinity, huge or infinite -> zero
+  const bool tiny = mag < 0x00100000u, huge = mag - 0x7fd00000u <= 0x00200000u;
+  const unsigned xh = tiny ? (sgn | 0x7ff00000u) : huge ? sgn : (unsigned)__double2hiint(x);
+  return __hiloint2double((int)xh, tiny || huge ? 0 : __double2loint(x));
 }
 #endif
 

@@ -625,7 +625,7 @@ __global__ void __launch_bounds__(BS, MINB) integrate_kernel(StepArgs a) {
           const float e = cvt<float>(fma(-2.0, k2[i], k1[i]) + xs[i]);
           const float ym = fmaxf(fabsf(cvt<float>(y[i])), fabsf(cvt<float>(y1[i])));
           const float sc = fmaxf(fmaf(rtol, ym, cvt<float>(a.atol[i])), 1e-30f);
-          const float r = fabsf(e) * __frcp_rn(sc);
+          const float r = fabsf(e) * rcp<float>(sc);
           if (!(r <= nf)) nf = r;  // NaN propagates
         }
         norm = nf * (cvt<float>(hh) * (1.0f / 6.0f));

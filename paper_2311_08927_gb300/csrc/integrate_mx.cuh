@@ -68,7 +68,7 @@ __device__ __forceinline__ float solve_h2_f32(const H2Bal<float>& e, float guess
     const float E = h2_eval<float>(e, S, dE);
     cnt.h2++;
     if (!(fabsf(E) <= fabsf(prevE)) || !(dE < 0.0f)) break;
-    const float dS = E * __frcp_rn(dE);
+    const float dS = E * rcp<float>(dE);
     const float Sn = S - dS;
     if (!(Sn > 0.0f) || !(Sn < 1e30f)) break;
     if (fabsf(dS) <= 1e-6f * Sn || E == 0.0f) return Sn;
@@ -275,7 +275,7 @@ __global__ void __launch_bounds__(BS, MINB) integrate_mx_kernel(StepArgs a) {
     // S_h2 leaves W_d: dS_h2/dy = -(J_h2,j + u_h2 v_j) / J_h2,h2 from its
     // row, g times its column becomes the second Sherman-Morrison vector
     {
-      const float rjj = __frcp_rn(zh[iS_h2]);
+      const float rjj = rcp<float>(zh[iS_h2]);
 #pragma unroll
       for (int j = 0; j < NS; ++j)
         zh[j] = (sp::slot(iS_h2, j) >= 0 && j != iS_h2) ? -zh[j] * rjj : 0.0f;
@@ -303,7 +303,7 @@ __global__ void __launch_bounds__(BS, MINB) integrate_mx_kernel(StepArgs a) {
 #pragma unroll
       for (int j = 0; j < NS; ++j) s2 = fmaf(zh[j], p2[j], s2);
       const float delta2 = 1.0f - s2;
-      inv_delta2 = __frcp_rn(delta2);
+      inv_delta2 = rcp<float>(delta2);
       piv_ok = piv_ok && isfinite(delta2) && delta2 != 0.0f &&
                fabsf(delta2) >= float(kPivTau) * fmaxf(1.0f, fabsf(s2));
     }
@@ -447,7 +447,7 @@ __global__ void __launch_bounds__(BS, MINB) integrate_mx_kernel(StepArgs a) {
           const float e = ed.hi + ed.lo;
           const float ym = fmaxf(fabsf(ys[i]), fabsf(y1s[i]));
           const float sc = fmaxf(fmaf(rtol, ym, f32(a.atol[i])), 1e-30f);
-          const float r = fabsf(e) * __frcp_rn(sc);
+          const float r = fabsf(e) * rcp<float>(sc);
           if (!(r <= nf)) nf = r;  // NaN propagates
         }
         norm = nf * (f32(hh) * (1.0f / 6.0f));
