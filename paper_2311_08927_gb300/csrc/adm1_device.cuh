@@ -13,6 +13,7 @@
 #pragma once
 #include <cmath>
 #include <cstdint>
+#include <cstring>
 
 #include "model.h"
 
@@ -237,28 +238,70 @@ struct AcidBase {
   double rS;     // 1/S_H
 };
 
-// E(S) and dE/dS of Eq. 7 from the reciprocals rS = 1/S and r = 1/(K_a + S)
-// for IN, co2, ac, pro, bu, va.
-template <class F>
-CHAD_HD F charge_terms(const DigConst& c, const PartConst& q, const double* y, F S, F rS,
-                       const F* r, F& dEdS) {
-  const F nh3 = F(q.K_a_IN) * F(y[iS_IN]) * r[0];
-  const F hco3 = F(q.K_a_co2) * F(y[iS_IC]) * r[1];
-  const F ac = F(c.K_a_ac) * F(y[iS_ac]) * r[2] * F(1.0 / kVfaCod_ac);
-  const F pro = F(c.K_a_pro) * F(y[iS_pro]) * r[3] * F(1.0 / kVfaCod_pro);
-  const F bu = F(c.K_a_bu) * F(y[iS_bu]) * r[4] * F(1.0 / kVfaCod_bu);
-  const F va = F(c.K_a_va) * F(y[iS_va]) * r[5] * F(1.0 / kVfaCod_va);
-  const F kw = F(q.K_w) * rS;
-  dEdS = F(1.0) + kw * rS + nh3 * r[0] + hco3 * r[1] + ac * r[2] + pro * r[3] + bu * r[4] +
-         va * r[5];
-  return (F(y[iS_cat]) - F(y[iS_an])) + (F(y[iS_IN]) - nh3) + S - hco3 - ac - pro - bu - va - kw;
-}
+struct NewtonCounters {
+  int iters;
+  int fallbacks;
+  int failed;
+};
 
-// E(S) and dE/dS; fills the reciprocals used by the Jacobian.  Templated
-// on the scalar type only so that its operations can be counted on the host.
+// The bit pattern of a double, its magnitude's pattern, and the high word of
+// the latter: finite magnitudes order like their patterns, and on the GPU an
+// FP64 compare takes an FP64 pipe slot where an integer compare does not.
+CHAD_HD long long bits64(double x) {
+#ifdef __CUDA_ARCH__
+  return __double_as_longlong(x);
+#else
+  long long b;
+  memcpy(&b, &x, sizeof(b));
+  return b;
+#endif
+}
+CHAD_HD long long mag64(double x) { return bits64(x) & 0x7fffffffffffffffll; }
+CHAD_HD int maghi(double x) { return (int)(mag64(x) >> 32); }
+constexpr long long kInfBits = 0x7ff0000000000000ll;
+CHAD_HD bool pos_finite(double x) { return (unsigned long long)bits64(x) - 1ull < (unsigned long long)kInfBits - 1ull; }
+// |t| <= 2^-18 |S| to within the piecewise-linear log2 of the patterns (6 %)
+CHAD_HD bool third_order_close(double t, double S) { return maghi(t) + (18 << 20) <= maghi(S); }
+
+// Eq. 7 with the products that do not change with S_H formed once per solve:
+//   E(S) = base + S - sum_k P_k / (K_k + S) - K_w / S
+// over IN, co2, ac, pro, bu, va (P = K_a times the concentration in charge
+// equivalents).
 template <class F>
-CHAD_HD F charge_E_t(const DigConst& c, const PartConst& q, const double* y, F S, F* r, F& rS,
-                     F& dEdS) {
+struct ChargeBalT {
+  F base, P[6];
+};
+using ChargeBal = ChargeBalT<double>;
+template <class F>
+CHAD_HD void charge_bal(const DigConst& c, const PartConst& q, const double* y, ChargeBalT<F>& e) {
+  e.base = (F(y[iS_cat]) - F(y[iS_an])) + F(y[iS_IN]);
+  e.P[0] = F(q.K_a_IN) * F(y[iS_IN]);
+  e.P[1] = F(q.K_a_co2) * F(y[iS_IC]);
+  e.P[2] = F(c.K_a_ac) * F(y[iS_ac]) * F(1.0 / kVfaCod_ac);
+  e.P[3] = F(c.K_a_pro) * F(y[iS_pro]) * F(1.0 / kVfaCod_pro);
+  e.P[4] = F(c.K_a_bu) * F(y[iS_bu]) * F(1.0 / kVfaCod_bu);
+  e.P[5] = F(c.K_a_va) * F(y[iS_va]) * F(1.0 / kVfaCod_va);
+}
+// E and dE/dS from the reciprocals rS = 1/S and r_k = 1/(K_k + S).  The
+// routines of the balance are templates on the scalar type so that their
+// operations can be counted on the host.
+template <class F>
+CHAD_HD F charge_sums(const ChargeBalT<F>& e, F K_w, F S, F rS, const F* r, F& dEdS) {
+  const F kw = K_w * rS;
+  F E = (e.base - kw) + S, d = F(1.0) + kw * rS;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    const F t = e.P[k] * r[k];
+    E = E - t;
+    d = d + t * r[k];
+  }
+  dEdS = d;
+  return E;
+}
+// E and dE/dS at S with the reciprocals.
+template <class F>
+CHAD_HD F charge_eval(const DigConst& c, const PartConst& q, const ChargeBalT<F>& e, F S, F* r,
+                      F& rS, F& dEdS) {
   rS = rcp<F>(S);
   r[0] = rcp<F>(F(q.K_a_IN) + S);
   r[1] = rcp<F>(F(q.K_a_co2) + S);
@@ -266,37 +309,34 @@ CHAD_HD F charge_E_t(const DigConst& c, const PartConst& q, const double* y, F S
   r[3] = rcp<F>(F(c.K_a_pro) + S);
   r[4] = rcp<F>(F(c.K_a_bu) + S);
   r[5] = rcp<F>(F(c.K_a_va) + S);
-  return charge_terms<F>(c, q, y, S, rS, r, dEdS);
+  return charge_sums<F>(e, F(q.K_w), S, rS, r, dEdS);
 }
-
-CHAD_HD double charge_E(const DigConst& c, const PartConst& q, const double* y, double S,
-                        AcidBase& ab) {
-  double r[6];
-  const double E = charge_E_t<double>(c, q, y, S, r, ab.rS, ab.dEdS);
-  ab.r_IN = r[0];
-  ab.r_co2 = r[1];
-  ab.r_ac = r[2];
-  ab.r_pro = r[3];
-  ab.r_bu = r[4];
-  ab.r_va = r[5];
-  return E;
-}
-
-// Move the reciprocals of charge_E_t from S to S + d to first order,
-// 1/(K + S + d) = r / (1 + r d) ~ r (1 - r d) with relative error (r d)^2,
-// and recompute dE/dS from them.  Templated for operation counting.
+// Chebyshev's third-order correction at a Newton update t = E inv, inv =
+// 1/E': the move d of the root, -t + t^2 h / E' with h = -E''/2.
 template <class F>
-CHAD_HD void root_shift_t(const DigConst& c, const PartConst& q, const double* y, F S, F d, F* r,
-                          F& rS, F& dEdS) {
-  rS = rS - rS * rS * d;
+CHAD_HD F charge_step(const ChargeBalT<F>& e, F K_w, F rS, const F* r, F t, F inv) {
+  F h = K_w * rS * (rS * rS);
 #pragma unroll
-  for (int k = 0; k < 6; ++k) r[k] = r[k] - r[k] * r[k] * d;
-  charge_terms<F>(c, q, y, S + d, rS, r, dEdS);
+  for (int k = 0; k < 6; ++k) h = h + e.P[k] * r[k] * (r[k] * r[k]);
+  return t * (t * (h * inv)) - t;
 }
-CHAD_HD void root_shift(const DigConst& c, const PartConst& q, const double* y, AcidBase& ab,
-                        double S, double d) {
-  double r[6] = {ab.r_IN, ab.r_co2, ab.r_ac, ab.r_pro, ab.r_bu, ab.r_va};
-  root_shift_t<double>(c, q, y, S, d, r, ab.rS, ab.dEdS);
+// The reciprocals moved from S to S + d to second order in x = r d,
+// 1/(K + S + d) = r / (1 + x) = r (1 - x + x^2 - ..), and dE/dS there.
+template <class F>
+CHAD_HD void charge_move(const ChargeBalT<F>& e, F K_w, F S, F d, F* r, F& rS, F& dEdS) {
+  F x = rS * d;
+  rS = rS + rS * (x * x - x);
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    x = r[k] * d;
+    r[k] = r[k] + r[k] * (x * x - x);
+  }
+  charge_sums<F>(e, K_w, S + d, rS, r, dEdS);
+}
+CHAD_HD void charge_fill(AcidBase& ab, double SH, double rS, const double* r, double dEdS) {
+  ab.SH = SH;
+  ab.dEdS = dEdS;
+  ab.rS = rS;
   ab.r_IN = r[0];
   ab.r_co2 = r[1];
   ab.r_ac = r[2];
@@ -304,129 +344,127 @@ CHAD_HD void root_shift(const DigConst& c, const PartConst& q, const double* y, 
   ab.r_bu = r[4];
   ab.r_va = r[5];
 }
-
-struct NewtonCounters {
-  int iters;
-  int fallbacks;
-  int failed;
-};
 
 // Newton from `guess` without a fallback: true if it converged within
-// max_iters with |E| <= max_resid at the returned root (ab then describes it).
-// E is increasing and concave, Newton converges quadratically with a
+// max_iters with |E| <= max_resid at the returned root (ab then describes
+// it).  E is increasing and concave, Newton converges quadratically with a
 // relative contraction factor below 1 near the root: an update below 1e-8
 // relative leaves the new iterate within ~1e-16 of the root.
 __host__ __device__ inline bool newton_only(const DigConst& c, const PartConst& q,
                                             const double* y, double guess, int max_iters,
                                             double max_resid, AcidBase& ab, int& iters) {
+  ChargeBal cb;
+  charge_bal<double>(c, q, y, cb);
   double S = (guess > 0.0 && isfinite(guess)) ? guess : 1e-7;
-  double prevE = INFINITY;
-  for (int it = 0; it < max_iters; ++it) {
-    const double E = charge_E(c, q, y, S, ab);
+  double prevE = INFINITY, Ec = INFINITY;
+  bool last = false;
+  for (int it = 0;; ++it) {
+    double r[6], rS, dE;
+    const double E = charge_eval<double>(c, q, cb, S, r, rS, dE);
+    if (last) {  // at the root: the residual bound
+      charge_fill(ab, S, rS, r, dE);
+      return fabs(E) <= max_resid || Ec <= max_resid;
+    }
+    if (it >= max_iters) return false;
     iters++;
     if (!isfinite(E) || fabs(E) > fabs(prevE)) return false;
-    const double dS = E * rcp<double>(ab.dEdS);
+    const double dS = E * rcp<double>(dE);
     const double Sn = S - dS;
     if (!(Sn > 0.0) || !isfinite(Sn)) return false;
-    if (fabs(dS) <= 1e-8 * Sn || fabs(E) <= 1e-15) {
-      ab.SH = Sn;
-      if (max_resid < INFINITY) {  // a residual bound is asked for: evaluate at the root
-        const double Ef = charge_E(c, q, y, Sn, ab);
-        return fabs(Ef) <= max_resid || fabs(E) <= max_resid;
-      }
-      // Otherwise move the reciprocals 1/S and 1/(K_a + S) to the root to
-      // first order; |r dS| <= 1e-8, so their relative error (r dS)^2 is at
-      // the FP64 rounding level, and dE/dS follows from them.
-      root_shift(c, q, y, ab, S, -dS);
-      return true;
-    }
+    last = fabs(dS) <= 1e-8 * Sn || fabs(E) <= 1e-15;
+    Ec = fabs(E);
     prevE = E;
     S = Sn;
   }
-  return false;
 }
 
-// Newton from `guess`; an iterate leaving (0, inf) or a growing |E| switches
-// to bisection on [1e-14, 1] (geometric midpoint, at most 200 halvings).
-// The same iterates as newton_only followed by the bisection, written as one
-// loop around a single evaluation of Eq. 7: each evaluation inlines seven
-// reciprocals, and one copy of it instead of seven keeps the integrator's
-// code within reach of the instruction cache.
+// Root of Eq. 7: Newton from `guess`; an iterate leaving (0, inf) or a
+// growing |E| switches to a bracket on [1e-14, 1].  One loop around a single
+// evaluation of Eq. 7: each evaluation inlines seven reciprocals, and one
+// copy keeps the integrator's code within reach of the instruction cache.
+//   * A Newton update t with |t| <= 2^-18 S ends the solve with the
+//     third-order step of Chebyshev, S - t + t^2 h / E' with h = -E''/2 =
+//     sum P r^3 + K_w / S^3: |E''/E'| <= 2/S and its higher relatives bound
+//     the remainder by a few (t/S)^3, below 1e-16.  The reciprocals move
+//     with the root, 1/(K + S + d) = r (1 - x + x^2) with x = r d and
+//     relative error x^3.  Plain Newton would need another evaluation (75
+//     FP64 instructions) in nearly every warp, since some lane's tangent
+//     guess is off by more than 1e-8.
+//   * Bracket: geometric midpoints halve its ratio's logarithm until
+//     hi <= 4 lo, then Newton inside it (E is increasing and concave: from
+//     the left Newton climbs to the root without passing it).  A dozen
+//     evaluations, where bisection to the last bit took over fifty.
 __host__ __device__ inline void solve_SH(const DigConst& c, const PartConst& q, const double* y,
                                          double guess, int max_iters, AcidBase& ab,
                                          NewtonCounters& nc) {
-  enum { kNewton, kLo, kHi, kBisect, kFinal };
-  const double start = (guess > 0.0 && isfinite(guess)) ? guess : 1e-7;
+  enum { kNewton, kLo, kHi, kBracket, kFinal };
+  ChargeBal cb;
+  charge_bal<double>(c, q, y, cb);
+  const double start = pos_finite(guess) ? guess : 1e-7;
   int phase = max_iters > 0 ? kNewton : kLo;
   if (phase == kLo) nc.fallbacks++;
   double S = phase == kNewton ? start : kSH_lo;  // point of the next evaluation
-  double prevE = INFINITY, lo = kSH_lo, hi = kSH_hi, elo = 0.0;
+  long long prevE = kInfBits;
+  double lo = kSH_lo, hi = kSH_hi;
+  bool lo_neg = false;
   int it = 0;
   for (;;) {
-    const double E = charge_E(c, q, y, S, ab);
-    if (phase == kFinal) {
-      ab.SH = S;
-      return;
-    }
-    if (phase == kNewton) {
-      nc.iters++;
-      bool fail = !isfinite(E) || fabs(E) > fabs(prevE);
-      if (!fail) {
-        const double dS = E * rcp<double>(ab.dEdS);
-        const double Sn = S - dS;
-        fail = !(Sn > 0.0) || !isfinite(Sn);
-        if (!fail && (fabs(dS) <= 1e-8 * Sn || fabs(E) <= 1e-15)) {
-          // converged: move the reciprocals 1/S and 1/(K_a + S) to the root
-          // to first order (|r dS| <= 1e-8: relative error at the FP64
-          // rounding level) and dE/dS with them
-          ab.SH = Sn;
-          root_shift(c, q, y, ab, S, -dS);
-          return;
-        }
+    double r[6], rS, dE;
+    const double E = charge_eval<double>(c, q, cb, S, r, rS, dE);
+    const double inv = rcp<double>(dE);
+    const double t = E * inv;
+    bool done = phase == kFinal;
+    double d = 0.0;
+    if (phase == kNewton || phase == kBracket) {
+      const long long mE = mag64(E);
+      const bool close = mE < kInfBits && third_order_close(t, S);
+      if (phase == kNewton) nc.iters++;
+      if (close && !(phase == kNewton && mE > prevE)) {
+        d = charge_step<double>(cb, q.K_w, rS, r, t, inv);
+        done = true;
+      } else if (phase == kNewton) {
+        const double Sn = S - t;
+        bool fail = mE >= kInfBits || mE > prevE || !pos_finite(Sn);
         if (!fail) {
-          prevE = E;
+          prevE = mE;
           S = Sn;
           fail = ++it >= max_iters;
         }
+        if (fail) {
+          nc.fallbacks++;
+          phase = kLo;
+          S = lo;
+        }
+      } else {
+        ++it;
+        if (bits64(E) < 0) lo = S; else hi = S;
+        const double mid = sqrt(lo * hi), Sn = S - t;
+        if (it >= 200 || !(mid > lo && mid < hi)) {
+          phase = kFinal;
+          S = mid;
+        } else {
+          S = hi <= 4.0 * lo && Sn > lo && Sn < hi ? Sn : mid;
+        }
       }
-      if (fail) {
-        nc.fallbacks++;
-        phase = kLo;
-        S = lo;
-      }
-      continue;
-    }
-    if (phase == kLo) {
-      elo = E;
+    } else if (phase == kLo) {
+      lo_neg = E < 0.0;
       phase = kHi;
       S = hi;
-      continue;
-    }
-    if (phase == kHi) {
-      if (!(elo < 0.0 && E > 0.0)) {  // no sign change: keep the guess
+    } else if (phase == kHi) {
+      if (!(lo_neg && E > 0.0)) {  // no sign change: keep the guess
         nc.failed = 1;
         phase = kFinal;
         S = start;
-        continue;
-      }
-      phase = kBisect;
-      it = 0;
-    } else {  // kBisect: E at the midpoint S
-      ++it;
-      if (E == 0.0) {
-        lo = hi = S;
-      } else if (E < 0.0) {
-        lo = S;
       } else {
-        hi = S;
+        phase = kBracket;
+        it = 0;
+        S = sqrt(lo * hi);
       }
     }
-    const double mid = sqrt(lo * hi);
-    if (lo == hi || it >= 200 || !(mid > lo && mid < hi)) {
-      phase = kFinal;
-      S = sqrt(lo * hi);
-    } else {
-      S = mid;
+    if (done) {
+      charge_move<double>(cb, q.K_w, S, d, r, rS, dE);
+      charge_fill(ab, S + d, rS, r, dE);
+      return;
     }
   }
 }
@@ -474,36 +512,68 @@ CHAD_HD void hill(R S, R invK, R n, int ni, R& I, R& dI) {
 // with P >= 0: E decreases in S and the root is unique.
 template <class F>
 struct H2Bal {
-  F C0, Pfa, Pc4, Ppro, Ph2, kD, Kfa, Kc4, Kpro, Kh2;
+  F C0, PKfa, PKc4, PKpro, Ph2, kD, Kfa, Kc4, Kpro, Kh2;  // PK = P K
 };
 
+// Factors of the rates that do not hold S_h2 (Eq. 3-6 inhibitions and Monod
+// terms): formed once per evaluation point and shared by the Eq. 8 balance
+// and the rates, ten reciprocals and about 60 operations fewer than forming
+// them in both.  B5 and B12 carry the Arrhenius factor.  The FP64 forms are
+// bound by the FP64 pipe, one warp instruction per 64 cycles and
+// sub-partition, so each instruction saved counts: with the partials below
+// and the products of structural zeros left out, 100,000 particles in the
+// shared-headspace cylinder take 54.5 ms instead of 58.0, ten fixed substeps
+// of 111,000 particles 8.54 instead of 9.18.
+template <class R>
+struct Factors {
+  R Ipaa, dIpaa, Iph2, dIph2;  // pH inhibitions (the aa form also of su, fa, c4, pro)
+  R rIN, IIN;
+  R rsu, raa, rfs, rva, rbu, rpo;  // 1/(K_S + S)
+  R msu, maa, mfa, mva, mbu, mpo;  // Monod terms
+  R rden, gva, gbu;                // c4 uptake split
+  R B5, B12;                       // arr I_pH I_IN
+};
+
+template <class R, class DC, class PQ, class Y>
+CHAD_HD void factors(const DC& c, const PQ& q, const Y* y, const AcidBase& ab, Factors<R>& k) {
+  hill<R>(R(ab.SH), R(c.inv_K_pH_aa), R(c.n_aa), c.ni_aa, k.Ipaa, k.dIpaa);
+  hill<R>(R(ab.SH), R(c.inv_K_pH_h2), R(c.n_h2), c.ni_h2, k.Iph2, k.dIph2);
+  const R S_IN = R(y[iS_IN]), S_va = R(y[iS_va]), S_bu = R(y[iS_bu]);
+  k.rIN = rcp<R>(S_IN + R(c.K_S_IN));
+  k.IIN = S_IN * k.rIN;
+  k.rsu = rcp<R>(R(c.K_S_su) + R(y[iS_su]));
+  k.raa = rcp<R>(R(c.K_S_aa) + R(y[iS_aa]));
+  k.rfs = rcp<R>(R(c.K_S_fa) + R(y[iS_fa]));
+  k.rva = rcp<R>(R(c.K_S_c4) + S_va);
+  k.rbu = rcp<R>(R(c.K_S_c4) + S_bu);
+  k.rpo = rcp<R>(R(c.K_S_pro) + R(y[iS_pro]));
+  k.msu = R(y[iS_su]) * k.rsu;
+  k.maa = R(y[iS_aa]) * k.raa;
+  k.mfa = R(y[iS_fa]) * k.rfs;
+  k.mva = S_va * k.rva;
+  k.mbu = S_bu * k.rbu;
+  k.mpo = R(y[iS_pro]) * k.rpo;
+  k.rden = rcp<R>(S_bu + S_va + R(kC4Guard));
+  k.gva = S_va * k.rden;
+  k.gbu = S_bu * k.rden;
+  const R aN = R(q.arr) * k.IIN;
+  k.B5 = k.Ipaa * aN;
+  k.B12 = k.Iph2 * aN;
+}
+
 template <class F, class DC, class PQ, class Y>
-CHAD_HD void h2_coeffs(const DC& c, const PQ& q, const Y* y, F D, const AcidBase& ab,
+CHAD_HD void h2_coeffs(const DC& c, const PQ& q, const Y* y, F D, const Factors<F>& k,
                        H2Bal<F>& e) {
-  const F a = F(q.arr);
-  F Ipaa, dIpaa, Iph2, dIph2;
-  hill<F>(F(ab.SH), F(c.inv_K_pH_aa), F(c.n_aa), c.ni_aa, Ipaa, dIpaa);
-  hill<F>(F(ab.SH), F(c.inv_K_pH_h2), F(c.n_h2), c.ni_h2, Iph2, dIph2);
-  const F S_IN = F(y[iS_IN]);
-  const F IIN = S_IN * rcp<F>(S_IN + F(c.K_S_IN));
-  const F msu = F(y[iS_su]) * rcp<F>(F(c.K_S_su) + F(y[iS_su]));
-  const F maa = F(y[iS_aa]) * rcp<F>(F(c.K_S_aa) + F(y[iS_aa]));
-  const F mfa = F(y[iS_fa]) * rcp<F>(F(c.K_S_fa) + F(y[iS_fa]));
-  const F mva = F(y[iS_va]) * rcp<F>(F(c.K_S_c4) + F(y[iS_va]));
-  const F mbu = F(y[iS_bu]) * rcp<F>(F(c.K_S_c4) + F(y[iS_bu]));
-  const F mpo = F(y[iS_pro]) * rcp<F>(F(c.K_S_pro) + F(y[iS_pro]));
-  const F rden = rcp<F>(F(y[iS_bu]) + F(y[iS_va]) + F(kC4Guard));
-  const F gva = F(y[iS_va]) * rden, gbu = F(y[iS_bu]) * rden;
-  const F B5 = Ipaa * IIN, B12 = Iph2 * IIN;
-  const F r4 = F(c.k_m_su) * a * F(y[iX_su]) * msu * B5;
-  const F r5 = F(c.k_m_aa) * a * F(y[iX_aa]) * maa * B5;
   const F kLa = F(c.k_La);
   const F KH2 = F(q.K_H_h2) * F(q.RT);
-  e.C0 = D * F(c.y_in[iS_h2]) + F(c.su_h2) * r4 + F(c.aa_h2) * r5 + kLa * KH2 * F(y[iG_h2]);
-  e.Pfa = F(c.fa_h2) * F(c.k_m_fa) * a * F(y[iX_fa]) * mfa * B5;
-  e.Pc4 = (F(c.va_h2) * mva * gva + F(c.bu_h2) * mbu * gbu) * F(c.k_m_c4) * a * F(y[iX_c4]) * B5;
-  e.Ppro = F(c.pro_h2) * F(c.k_m_pro) * a * F(y[iX_pro]) * mpo * B5;
-  e.Ph2 = F(c.k_m_h2) * a * F(y[iX_h2]) * B12;
+  const F r4 = F(c.k_m_su) * F(y[iX_su]) * k.msu;
+  const F r5 = F(c.k_m_aa) * F(y[iX_aa]) * k.maa;
+  e.C0 = D * F(c.y_in[iS_h2]) + (F(c.su_h2) * r4 + F(c.aa_h2) * r5) * k.B5 + kLa * KH2 * F(y[iG_h2]);
+  e.PKfa = F(c.fa_h2) * (F(c.k_m_fa) * F(y[iX_fa]) * k.mfa) * k.B5 * F(c.K_I_h2_fa);
+  e.PKc4 = (F(c.va_h2) * (k.mva * k.gva) + F(c.bu_h2) * (k.mbu * k.gbu)) *
+           (F(c.k_m_c4) * F(y[iX_c4])) * k.B5 * F(c.K_I_h2_c4);
+  e.PKpro = F(c.pro_h2) * (F(c.k_m_pro) * F(y[iX_pro]) * k.mpo) * k.B5 * F(c.K_I_h2_pro);
+  e.Ph2 = F(c.k_m_h2) * F(y[iX_h2]) * k.B12;
   e.kD = kLa + D;
   e.Kfa = F(c.K_I_h2_fa);
   e.Kc4 = F(c.K_I_h2_c4);
@@ -511,41 +581,45 @@ CHAD_HD void h2_coeffs(const DC& c, const PQ& q, const Y* y, F D, const AcidBase
   e.Kh2 = F(c.K_S_h2);
 }
 
-// E(S) and dE/dS of Eq. 8 from the coefficients.
+// E(S) and dE/dS of Eq. 8 from the coefficients; h (may be null) receives
+// E''/2.
 template <class F>
-CHAD_HD F h2_eval(const H2Bal<F>& e, F S, F& dE) {
+CHAD_HD F h2_eval(const H2Bal<F>& e, F S, F& dE, F* h = nullptr) {
   const F rfa = rcp<F>(e.Kfa + S), rc4 = rcp<F>(e.Kc4 + S), rpr = rcp<F>(e.Kpro + S);
   const F rh = rcp<F>(e.Kh2 + S);
-  const F Ifa = e.Kfa * rfa, Ic4 = e.Kc4 * rc4, Ipr = e.Kpro * rpr;
-  dE = F(0) - (e.Pfa * Ifa * rfa + e.Pc4 * Ic4 * rc4 + e.Ppro * Ipr * rpr +
-               e.Ph2 * e.Kh2 * rh * rh + e.kD);
-  return e.C0 + e.Pfa * Ifa + e.Pc4 * Ic4 + e.Ppro * Ipr - e.Ph2 * S * rh - e.kD * S;
+  const F tfa = e.PKfa * rfa, tc4 = e.PKc4 * rc4, tpr = e.PKpro * rpr, th = e.Ph2 * rh;
+  const F dfa = tfa * rfa, dc4 = tc4 * rc4, dpr = tpr * rpr, dh = th * (e.Kh2 * rh);
+  dE = F(0) - (dfa + dc4 + dpr + dh + e.kD);
+  if (h) *h = dfa * rfa + dc4 * rc4 + dpr * rpr + dh * rh;
+  return e.C0 + tfa + tc4 + tpr - (th + e.kD) * S;
 }
 
-// Root of Eq. 8 by Newton from the guess: an update below 1e-8 relative
-// leaves the next iterate within ~1e-16 (quadratic convergence).  An iterate
-// leaving (0, inf), a growing |E| or a non-negative slope switches to
-// bisection on [0, hi], hi doubled from the guess until E(hi) <= 0 (E
-// decreases, and E(0) >= 0: at S = 0 nothing removes hydrogen but the
-// transfer from a gas that holds some).
+// Root of Eq. 8 by Newton from the guess, ended by Chebyshev's third-order
+// step as in solve_SH (|E''/E'| <= 2/S here too).  An iterate leaving (0,
+// inf), a growing |E| or a non-negative slope switches to bisection on [0,
+// hi], hi doubled from the guess until E(hi) <= 0 (E decreases, and E(0) >=
+// 0: at S = 0 nothing removes hydrogen but the transfer from a gas that
+// holds some).
 __host__ __device__ inline double solve_h2(const H2Bal<double>& e, double guess, int max_iters,
                                            NewtonCounters& nc) {
-  double S = (guess > 0.0 && isfinite(guess)) ? guess : 1e-8;
-  double prevE = INFINITY;
+  double S = pos_finite(guess) ? guess : 1e-8;
+  long long prevE = kInfBits;
   for (int it = 0; it < max_iters; ++it) {
-    double dE;
-    const double E = h2_eval<double>(e, S, dE);
+    double dE, h;
+    const double E = h2_eval<double>(e, S, dE, &h);
+    const long long mE = mag64(E);
     nc.iters++;
-    if (!isfinite(E) || fabs(E) > fabs(prevE) || !(dE < 0.0)) break;
-    const double dS = E * rcp<double>(dE);
-    const double Sn = S - dS;
-    if (!(Sn > 0.0) || !isfinite(Sn)) break;
-    if (fabs(dS) <= 1e-8 * Sn || E == 0.0) return Sn;
-    prevE = E;
+    if (mE >= kInfBits || mE > prevE || bits64(dE) >= 0 || mag64(dE) > kInfBits) break;
+    const double inv = rcp<double>(dE);
+    const double t = E * inv;
+    if (third_order_close(t, S)) return S - t - t * (t * (h * inv));
+    const double Sn = S - t;
+    if (!pos_finite(Sn)) break;
+    prevE = mE;
     S = Sn;
   }
   nc.fallbacks++;
-  double lo = 0.0, hi = fmax((guess > 0.0 && isfinite(guess)) ? guess : 0.0, 1e-12), dE;
+  double lo = 0.0, hi = fmax(pos_finite(guess) ? guess : 0.0, 1e-12), dE;
   int k = 0;
   while (k < 200 && h2_eval<double>(e, hi, dE) > 0.0) {
     hi *= 2.0;
@@ -553,7 +627,7 @@ __host__ __device__ inline double solve_h2(const H2Bal<double>& e, double guess,
   }
   if (k == 200) {
     nc.failed = 1;
-    return (guess > 0.0 && isfinite(guess)) ? guess : 1e-8;
+    return pos_finite(guess) ? guess : 1e-8;
   }
   for (int it = 0; it < 200; ++it) {
     const double mid = 0.5 * (lo + hi);
@@ -574,23 +648,22 @@ struct Rates {
   R s5, s6, s7, s8, s9, s10, s11, s12;                // wrt S_H
   R ddec[7];
   R dT8[2], dT9[2], dT10[2], sT10;
-  R qv, dqv;                                          // q_gas/V_gas, its dP derivative
+  R qv, qvs, dqv;                                     // q_gas/V_gas (qvs scaled), its dP derivative
   R P_h2, P_ch4, P_co2;                               // dP/dG
 };
 
+// k: the factors at y (factors()).  J: the partials too, multiplied by sc
+// (the FP64 forms take sc = -g, so that the Jacobian scatter yields -g J_d
+// and -g u): sc goes into the few factors that all partials of a process
+// share instead of multiplying each of some 60 partials.
 template <class R, bool J, class DC, class PQ>
-CHAD_HD void rates(const DC& c, const PQ& q, const R* y, const AcidBase& ab, Rates<R>& o) {
+CHAD_HD void rates(const DC& c, const PQ& q, const R* y, const AcidBase& ab, const Factors<R>& k,
+                   Rates<R>& o, R sc = R(1)) {
   const R a = R(q.arr);
   const R SH = R(ab.SH);
-  // inhibition factors (Eq. 3-6)
-  R Ipaa, dIpaa, Ipac, dIpac, Iph2, dIph2;
-  hill<R>(SH, R(c.inv_K_pH_aa), R(c.n_aa), c.ni_aa, Ipaa, dIpaa);
+  R Ipac, dIpac;
   hill<R>(SH, R(c.inv_K_pH_ac), R(c.n_ac), c.ni_ac, Ipac, dIpac);
-  hill<R>(SH, R(c.inv_K_pH_h2), R(c.n_h2), c.ni_h2, Iph2, dIph2);
   const R S_IN = y[iS_IN], S_h2 = y[iS_h2];
-  const R rIN = rcp<R>(S_IN + R(c.K_S_IN));
-  const R IIN = S_IN * rIN;
-  const R dIIN = R(c.K_S_IN) * rIN * rIN;
   const R rfa = rcp<R>(R(c.K_I_h2_fa) + S_h2), rc4 = rcp<R>(R(c.K_I_h2_c4) + S_h2);
   const R rpr = rcp<R>(R(c.K_I_h2_pro) + S_h2);
   const R Ih2fa = R(c.K_I_h2_fa) * rfa, Ih2c4 = R(c.K_I_h2_c4) * rc4, Ih2pro = R(c.K_I_h2_pro) * rpr;
@@ -606,37 +679,30 @@ CHAD_HD void rates(const DC& c, const PQ& q, const R* y, const AcidBase& ab, Rat
   o.r[1] = kch * y[iX_ch];
   o.r[2] = kpr * y[iX_pr];
   o.r[3] = kli * y[iX_li];
-  // Monod terms m = S/(K+S), dm = K/(K+S)^2
-  const R rsu = rcp<R>(R(c.K_S_su) + y[iS_su]), raa = rcp<R>(R(c.K_S_aa) + y[iS_aa]);
-  const R rfs = rcp<R>(R(c.K_S_fa) + y[iS_fa]), rva = rcp<R>(R(c.K_S_c4) + y[iS_va]);
-  const R rbu = rcp<R>(R(c.K_S_c4) + y[iS_bu]), rpo = rcp<R>(R(c.K_S_pro) + y[iS_pro]);
+  // uptakes: p = k_m X x Monod terms, the rate p B
   const R rac = rcp<R>(R(c.K_S_ac) + y[iS_ac]), rh2 = rcp<R>(R(c.K_S_h2) + S_h2);
-  const R msu = y[iS_su] * rsu, maa = y[iS_aa] * raa, mfa = y[iS_fa] * rfs, mva = y[iS_va] * rva;
-  const R mbu = y[iS_bu] * rbu, mpo = y[iS_pro] * rpo, mac = y[iS_ac] * rac, mh2 = S_h2 * rh2;
-  const R rden = rcp<R>(y[iS_bu] + y[iS_va] + R(kC4Guard));
-  const R gva = y[iS_va] * rden, gbu = y[iS_bu] * rden;
-
-  const R ksu = R(c.k_m_su) * a, kaa = R(c.k_m_aa) * a, kfa = R(c.k_m_fa) * a,
-          kc4 = R(c.k_m_c4) * a, kpo = R(c.k_m_pro) * a, kac = R(c.k_m_ac) * a,
-          kh2 = R(c.k_m_h2) * a;
-  const R B5 = Ipaa * IIN;
-  const R B7 = B5 * Ih2fa, B8 = B5 * Ih2c4, B10 = B5 * Ih2pro;
-  const R B11 = Ipac * IIN * Inh3, B12 = Iph2 * IIN;
-  const R A5 = ksu * y[iX_su], A6 = kaa * y[iX_aa], A7 = kfa * y[iX_fa], A8 = kc4 * y[iX_c4];
-  const R A10 = kpo * y[iX_pro], A11 = kac * y[iX_ac], A12 = kh2 * y[iX_h2];
-  o.r[4] = A5 * msu * B5;
-  o.r[5] = A6 * maa * B5;
-  o.r[6] = A7 * mfa * B7;
-  o.r[7] = A8 * mva * gva * B8;
-  o.r[8] = A8 * mbu * gbu * B8;
-  o.r[9] = A10 * mpo * B10;
-  o.r[10] = A11 * mac * B11;
-  o.r[11] = A12 * mh2 * B12;
+  const R mac = y[iS_ac] * rac, mh2 = S_h2 * rh2;
+  const R B7 = k.B5 * Ih2fa, B8 = k.B5 * Ih2c4, B10 = k.B5 * Ih2pro;
+  const R B11 = Ipac * (a * k.IIN) * Inh3;
+  const R A5 = R(c.k_m_su) * y[iX_su], A6 = R(c.k_m_aa) * y[iX_aa], A7 = R(c.k_m_fa) * y[iX_fa];
+  const R A8 = R(c.k_m_c4) * y[iX_c4], A10 = R(c.k_m_pro) * y[iX_pro], A11 = R(c.k_m_ac) * y[iX_ac];
+  const R A12 = R(c.k_m_h2) * y[iX_h2];
+  const R tva = k.mva * k.gva, tbu = k.mbu * k.gbu;
+  const R p5 = A5 * k.msu, p6 = A6 * k.maa, p7 = A7 * k.mfa, p8 = A8 * tva, p9 = A8 * tbu;
+  const R p10 = A10 * k.mpo, p11 = A11 * mac, p12 = A12 * mh2;
+  o.r[4] = p5 * k.B5;
+  o.r[5] = p6 * k.B5;
+  o.r[6] = p7 * B7;
+  o.r[7] = p8 * B8;
+  o.r[8] = p9 * B8;
+  o.r[9] = p10 * B10;
+  o.r[10] = p11 * B11;
+  o.r[11] = p12 * k.B12;
   R kd[7];
 #pragma unroll
-  for (int k = 0; k < 7; ++k) {
-    kd[k] = R(c.k_dec[k]) * a;
-    o.r[12 + k] = kd[k] * y[iX_su + k];
+  for (int i = 0; i < 7; ++i) {
+    kd[i] = R(c.k_dec[i]) * a;
+    o.r[12 + i] = kd[i] * y[iX_su + i];
   }
   // gas phase
   const R RT = R(q.RT);
@@ -653,65 +719,77 @@ CHAD_HD void rates(const DC& c, const PQ& q, const R* y, const AcidBase& ab, Rat
   o.r[21] = kLa * (y[iS_IC] * fco2 - KCO2 * y[iG_co2]);
 
   if (J) {
-    o.d1 = kdis; o.d2 = kch; o.d3 = kpr; o.d4 = kli;
+    o.d1 = kdis * sc; o.d2 = kch * sc; o.d3 = kpr * sc; o.d4 = kli * sc;
+    // scaled factors of the uptakes and their derivatives to S_IN (G) and S_H (H)
+    const R as = a * sc, aN = as * k.IIN;
+    const R dIIN = as * (R(c.K_S_IN) * k.rIN * k.rIN);
+    const R Bs = k.B5 * sc, G = k.Ipaa * dIIN, H = k.dIpaa * aN;
     // rho5: S_su, X_su, S_IN
-    o.d5[0] = A5 * (R(c.K_S_su) * rsu * rsu) * B5;
-    o.d5[1] = ksu * msu * B5;
-    o.d5[2] = A5 * msu * Ipaa * dIIN;
-    o.s5 = A5 * msu * dIpaa * IIN;
+    o.d5[0] = A5 * Bs * (R(c.K_S_su) * k.rsu * k.rsu);
+    o.d5[1] = R(c.k_m_su) * k.msu * Bs;
+    o.d5[2] = p5 * G;
+    o.s5 = p5 * H;
     // rho6: S_aa, X_aa, S_IN
-    o.d6[0] = A6 * (R(c.K_S_aa) * raa * raa) * B5;
-    o.d6[1] = kaa * maa * B5;
-    o.d6[2] = A6 * maa * Ipaa * dIIN;
-    o.s6 = A6 * maa * dIpaa * IIN;
-    // rho7: S_fa, X_fa, S_IN, S_h2
-    o.d7[0] = A7 * (R(c.K_S_fa) * rfs * rfs) * B7;
-    o.d7[1] = kfa * mfa * B7;
-    o.d7[2] = A7 * mfa * Ipaa * dIIN * Ih2fa;
-    o.d7[3] = -A7 * mfa * B5 * Ih2fa * rfa;   // dI/dS_h2 = -K/(K+S)^2 = -I r
-    o.s7 = A7 * mfa * dIpaa * IIN * Ih2fa;
+    o.d6[0] = A6 * Bs * (R(c.K_S_aa) * k.raa * k.raa);
+    o.d6[1] = R(c.k_m_aa) * k.maa * Bs;
+    o.d6[2] = p6 * G;
+    o.s6 = p6 * H;
+    // rho7: S_fa, X_fa, S_IN, S_h2 (dI/dS_h2 = -K/(K+S)^2 = -I r)
+    const R Bs7 = Bs * Ih2fa, p7i = p7 * Ih2fa;
+    o.d7[0] = A7 * Bs7 * (R(c.K_S_fa) * k.rfs * k.rfs);
+    o.d7[1] = R(c.k_m_fa) * k.mfa * Bs7;
+    o.d7[2] = p7i * G;
+    o.d7[3] = -p7i * Bs * rfa;
+    o.s7 = p7i * H;
     // rho8, rho9: S_va, S_bu, X_c4, S_IN, S_h2
-    const R rd2 = rden * rden;
+    const R rd2 = k.rden * k.rden;
     const R dgva_va = (y[iS_bu] + R(kC4Guard)) * rd2, dgva_bu = -y[iS_va] * rd2;
     const R dgbu_bu = (y[iS_va] + R(kC4Guard)) * rd2, dgbu_va = -y[iS_bu] * rd2;
-    const R dmva = R(c.K_S_c4) * rva * rva, dmbu = R(c.K_S_c4) * rbu * rbu;
-    o.d8[0] = A8 * B8 * (dmva * gva + mva * dgva_va);
-    o.d8[1] = A8 * B8 * mva * dgva_bu;
-    o.d8[2] = kc4 * mva * gva * B8;
-    o.d8[3] = A8 * mva * gva * Ipaa * dIIN * Ih2c4;
-    o.d8[4] = -A8 * mva * gva * B5 * Ih2c4 * rc4;
-    o.s8 = A8 * mva * gva * dIpaa * IIN * Ih2c4;
-    o.d9[0] = A8 * B8 * mbu * dgbu_va;
-    o.d9[1] = A8 * B8 * (dmbu * gbu + mbu * dgbu_bu);
-    o.d9[2] = kc4 * mbu * gbu * B8;
-    o.d9[3] = A8 * mbu * gbu * Ipaa * dIIN * Ih2c4;
-    o.d9[4] = -A8 * mbu * gbu * B5 * Ih2c4 * rc4;
-    o.s9 = A8 * mbu * gbu * dIpaa * IIN * Ih2c4;
+    const R dmva = R(c.K_S_c4) * k.rva * k.rva, dmbu = R(c.K_S_c4) * k.rbu * k.rbu;
+    const R Bs8 = Bs * Ih2c4, AB8 = A8 * Bs8, kB8 = R(c.k_m_c4) * Bs8, Bsr = Bs * rc4;
+    const R p8i = p8 * Ih2c4, p9i = p9 * Ih2c4;
+    o.d8[0] = AB8 * (dmva * k.gva + k.mva * dgva_va);
+    o.d8[1] = AB8 * (k.mva * dgva_bu);
+    o.d8[2] = kB8 * tva;
+    o.d8[3] = p8i * G;
+    o.d8[4] = -p8i * Bsr;
+    o.s8 = p8i * H;
+    o.d9[0] = AB8 * (k.mbu * dgbu_va);
+    o.d9[1] = AB8 * (dmbu * k.gbu + k.mbu * dgbu_bu);
+    o.d9[2] = kB8 * tbu;
+    o.d9[3] = p9i * G;
+    o.d9[4] = -p9i * Bsr;
+    o.s9 = p9i * H;
     // rho10: S_pro, X_pro, S_IN, S_h2
-    o.d10[0] = A10 * (R(c.K_S_pro) * rpo * rpo) * B10;
-    o.d10[1] = kpo * mpo * B10;
-    o.d10[2] = A10 * mpo * Ipaa * dIIN * Ih2pro;
-    o.d10[3] = -A10 * mpo * B5 * Ih2pro * rpr;
-    o.s10 = A10 * mpo * dIpaa * IIN * Ih2pro;
+    const R Bs10 = Bs * Ih2pro, p10i = p10 * Ih2pro;
+    o.d10[0] = A10 * Bs10 * (R(c.K_S_pro) * k.rpo * k.rpo);
+    o.d10[1] = R(c.k_m_pro) * k.mpo * Bs10;
+    o.d10[2] = p10i * G;
+    o.d10[3] = -p10i * Bs * rpr;
+    o.s10 = p10i * H;
     // rho11: S_ac, X_ac, S_IN (I_IN and free ammonia)
     const R dInh3 = -Inh3 * rnh;  // dI_nh3 / dS_nh3
-    o.d11[0] = A11 * (R(c.K_S_ac) * rac * rac) * B11;
-    o.d11[1] = kac * mac * B11;
-    o.d11[2] = A11 * mac * Ipac * (dIIN * Inh3 + IIN * dInh3 * r_nh3);
-    o.s11 = A11 * mac * IIN * (dIpac * Inh3 - Ipac * dInh3 * nh3 * R(ab.r_IN));
+    const R Bs11 = B11 * sc;
+    o.d11[0] = A11 * Bs11 * (R(c.K_S_ac) * rac * rac);
+    o.d11[1] = R(c.k_m_ac) * mac * Bs11;
+    o.d11[2] = p11 * (Ipac * (dIIN * Inh3 + aN * (dInh3 * r_nh3)));
+    o.s11 = p11 * (aN * (dIpac * Inh3 - Ipac * dInh3 * nh3 * R(ab.r_IN)));
     // rho12: S_h2, X_h2, S_IN
-    o.d12[0] = A12 * (R(c.K_S_h2) * rh2 * rh2) * B12;
-    o.d12[1] = kh2 * mh2 * B12;
-    o.d12[2] = A12 * mh2 * Iph2 * dIIN;
-    o.s12 = A12 * mh2 * dIph2 * IIN;
+    const R Bs12 = k.B12 * sc;
+    o.d12[0] = A12 * Bs12 * (R(c.K_S_h2) * rh2 * rh2);
+    o.d12[1] = R(c.k_m_h2) * mh2 * Bs12;
+    o.d12[2] = p12 * (k.Iph2 * dIIN);
+    o.s12 = p12 * (k.dIph2 * aN);
 #pragma unroll
-    for (int k = 0; k < 7; ++k) o.ddec[k] = kd[k];
-    // transfers
-    o.dT8[0] = kLa; o.dT8[1] = -kLa * KH2;
-    o.dT9[0] = kLa; o.dT9[1] = -kLa * KCH4;
-    o.dT10[0] = kLa * fco2; o.dT10[1] = -kLa * KCO2;
-    o.sT10 = kLa * y[iS_IC] * R(q.K_a_co2) * rco2 * rco2;
-    o.dqv = kpv * (R(2) * P - R(c.P_atm)) * invPa;
+    for (int i = 0; i < 7; ++i) o.ddec[i] = kd[i] * sc;
+    // transfers and gas outflow
+    const R kLs = kLa * sc, kps = kpv * invPa * sc;
+    o.dT8[0] = kLs; o.dT8[1] = -kLs * KH2;
+    o.dT9[0] = kLs; o.dT9[1] = -kLs * KCH4;
+    o.dT10[0] = kLs * fco2; o.dT10[1] = -kLs * KCO2;
+    o.sT10 = kLs * y[iS_IC] * (R(q.K_a_co2) * rco2 * rco2);
+    o.qvs = o.qv * sc;
+    o.dqv = kps * (R(2) * P - R(c.P_atm));
     o.P_h2 = P_h2; o.P_ch4 = P_ch4; o.P_co2 = P_co2;
   }
 }
@@ -765,29 +843,6 @@ CHAD_HD void stoich(const DC& c, const R* r, const R* dil, R* f) {
   f[iG_co2] = dil[iG_co2] + vr * r[21];
 }
 
-// Multiply every rate partial that enters the Jacobian (and u = df/dS_H) by
-// sc.  The FP64 form scales by -g before the Jacobian scatter, which then
-// yields -g J_d and -g u directly: W_d = I - g J_d needs only its diagonal
-// ones, instead of a multiply per stored slot.
-template <class R>
-CHAD_HD void scale_partials(Rates<R>& o, R sc) {
-  o.d1 *= sc; o.d2 *= sc; o.d3 *= sc; o.d4 *= sc;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) { o.d5[k] *= sc; o.d6[k] *= sc; o.d11[k] *= sc; o.d12[k] *= sc; }
-#pragma unroll
-  for (int k = 0; k < 4; ++k) { o.d7[k] *= sc; o.d10[k] *= sc; }
-#pragma unroll
-  for (int k = 0; k < 5; ++k) { o.d8[k] *= sc; o.d9[k] *= sc; }
-  o.s5 *= sc; o.s6 *= sc; o.s7 *= sc; o.s8 *= sc; o.s9 *= sc; o.s10 *= sc; o.s11 *= sc; o.s12 *= sc;
-#pragma unroll
-  for (int k = 0; k < 7; ++k) o.ddec[k] *= sc;
-#pragma unroll
-  for (int k = 0; k < 2; ++k) { o.dT8[k] *= sc; o.dT9[k] *= sc; o.dT10[k] *= sc; }
-  o.sT10 *= sc;
-  o.qv *= sc;
-  o.dqv *= sc;
-}
-
 // f(y): mass balances of Eq. 2 with the ADM1 stoichiometry
 template <class R, class DC>
 CHAD_HD void balances(const DC& c, const R* y, R D, const Rates<R>& o, R* f) {
@@ -838,7 +893,7 @@ CHAD_HD void jvp(const DC& c, const C* y, C D, const Rates<RO>& o, const RD* x, 
   RD dil[NS];
 #pragma unroll
   for (int i = 0; i < 26; ++i) dil[i] = -D * x[i];
-  const C qv = C(o.qv);
+  const C qv = C(o.qvs);
   const RD dq =
       C(o.dqv) * (C(o.P_h2) * x[iG_h2] + C(o.P_ch4) * x[iG_ch4] + C(o.P_co2) * x[iG_co2]);
   dil[iG_h2] = -x[iG_h2] * qv - y[iG_h2] * dq;
@@ -873,14 +928,21 @@ CHAD_HD void scat(JS Jm, int row, R coef, const int (&cols)[NC], const R (&d)[NC
 // With u_out == nullptr the full J = J_d + u v^T is assembled; otherwise only
 // the direct part J_d (S_H held fixed) goes into Jm and u = df/dS_H into
 // u_out, for the Sherman-Morrison solve of W = W_d - g u v^T.
-template <class Idx, class R, class JS, class DC, class PQ>
+// The sums start from -0, the identity of IEEE addition, so that the first
+// term of each slot costs no addition (0 + v would: it turns -0 into 0).
+// UNIT > 0: diagonal slots below UNIT start from 1 instead (with partials
+// and D scaled by -g the slots below UNIT then hold W_d = I - g J_d).
+template <class Idx, class R, int UNIT = 0, class JS, class DC, class PQ>
 CHAD_HD void jacobian(const DC& c, const PQ& q, const R* y, R D, const AcidBase& ab,
                       const Rates<R>& o, JS Jm, R* u_out = nullptr) {
   R u[NS];
 #pragma unroll
-  for (int i = 0; i < Idx::size; ++i) Jm[i] = R(0);
+  for (int i = 0; i < Idx::size; ++i) Jm[i] = R(-0.0);
 #pragma unroll
-  for (int i = 0; i < NS; ++i) u[i] = R(0);
+  for (int i = 0; i < NS; ++i) u[i] = R(-0.0);
+#pragma unroll
+  for (int i = 0; i < NS; ++i)
+    if (Idx::at(i, i) < UNIT) Jm[Idx::at(i, i)] = R(1);
 #pragma unroll
   for (int i = 0; i < 26; ++i) jadd<Idx>(Jm, i, i, -D);
   const R one = R(1), mone = R(-1);
@@ -1011,7 +1073,7 @@ CHAD_HD void jacobian(const DC& c, const PQ& q, const R* y, R D, const AcidBase&
     const R dP[3] = {o.P_h2, o.P_ch4, o.P_co2};
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      jadd<Idx>(Jm, g[a], g[a], -o.qv);
+      jadd<Idx>(Jm, g[a], g[a], -o.qvs);
       const R gq = y[g[a]] * o.dqv;
 #pragma unroll
       for (int b = 0; b < 3; ++b) jadd<Idx>(Jm, g[a], g[b], -gq * dP[b]);

@@ -87,13 +87,13 @@ __device__ __forceinline__ void newton(const DigConst& c, const PartConst& q, co
   SHg = ab.SH;
 }
 
-// S_h2 from Eq. 8 at y (S_H given by ab), Newton from *SH2g, which receives
+// S_h2 from Eq. 8 at y (S_H in the factors k), Newton from *SH2g, which receives
 // the root (algebraic S_h2 form).
 __device__ __forceinline__ void newton_h2(const DigConst& c, const PartConst& q, const double* y,
-                                          double D, const AcidBase& ab, double* SH2g,
+                                          double D, const Factors<double>& k, double* SH2g,
                                           int max_newton, Cnt& cnt) {
   H2Bal<double> e;
-  h2_coeffs<double>(c, q, y, D, ab, e);
+  h2_coeffs<double>(c, q, y, D, k, e);
   NewtonCounters nc{0, 0, 0};
   *SH2g = solve_h2(e, *SH2g, max_newton, nc);
   cnt.h2 += nc.iters;
@@ -112,12 +112,14 @@ __device__ __forceinline__ void eval_f(const DigConst& c, const PartConst& q, co
   RS yr[NS];
 #pragma unroll
   for (int i = 0; i < NS; ++i) yr[i] = RS(y[i]);
+  Factors<RS> k;
+  factors<RS>(c, q, yr, ab, k);
   if constexpr (H2A) {
-    newton_h2(c, q, y, D, ab, SH2g, max_newton, cnt);
+    newton_h2(c, q, y, D, k, SH2g, max_newton, cnt);
     yr[iS_h2] = RS(*SH2g);
   }
   Rates<RS> o;
-  rates<RS, false>(c, q, yr, ab, o);
+  rates<RS, false>(c, q, yr, ab, k, o);
   RS fr[NS];
   balances<RS>(c, yr, RS(D), o, fr);
 #pragma unroll
@@ -127,7 +129,7 @@ __device__ __forceinline__ void eval_f(const DigConst& c, const PartConst& q, co
 
 // f(y) in precision RS, J_d (sparse slots) and u = df/dS_H in precision R,
 // one Newton solve.  SCALE (FP64 form only, where R is RS): J_d and u come
-// out multiplied by jscale (the rate partials are scaled after f is formed).
+// out multiplied by jscale, and the slots below UNIT hold I + jscale J_d.
 // IX: the slot map of the Jacobian scatter (sp::Idx; with S_h2 algebraic
 // spa::Idx, with w an H2Split that takes S_h2's row and column apart).
 // The digester constants in the precision of the Jacobian evaluation.
@@ -146,20 +148,25 @@ struct DCSel<float> {
   }
 };
 
-template <class R, class RS, bool SCALE, bool H2A = false, class IX = sp::Idx, class W>
+template <class R, class RS, bool SCALE, bool H2A = false, class IX = sp::Idx, int UNIT = 0,
+          class W>
 __device__ __forceinline__ void eval_fj(const DigConst& c, const DigConstF* cf, const PartConst& q,
                                         const double* y, double D, double& SHg, int max_newton,
                                         Cnt& cnt, double* f, W w, R* u, Rates<R>& o,
                                         AcidBase& ab, R jscale, double* SH2g = nullptr) {
   const auto& cr = DCSel<R>::get(c, cf);
   newton(c, q, y, SHg, max_newton, cnt, ab);
-  if constexpr (H2A) newton_h2(c, q, y, D, ab, SH2g, max_newton, cnt);
   {
     R yr[NS];
 #pragma unroll
     for (int i = 0; i < NS; ++i) yr[i] = R(y[i]);
-    if constexpr (H2A) yr[iS_h2] = R(*SH2g);
-    rates<R, true>(cr, q, yr, ab, o);
+    Factors<R> k;
+    factors<R>(cr, q, yr, ab, k);
+    if constexpr (H2A) {
+      newton_h2(c, q, y, D, k, SH2g, max_newton, cnt);
+      yr[iS_h2] = R(*SH2g);
+    }
+    rates<R, true>(cr, q, yr, ab, k, o, SCALE ? jscale : R(1));
     if (std::is_same<R, RS>::value) {
       R fr[NS];
       balances<R>(cr, yr, R(D), o, fr);
@@ -168,8 +175,7 @@ __device__ __forceinline__ void eval_fj(const DigConst& c, const DigConstF* cf, 
       if constexpr (H2A) f[iS_h2] = 0.0;
     }
     if constexpr (SCALE) {
-      scale_partials<R>(o, jscale);
-      jacobian<IX, R>(cr, q, yr, R(D) * jscale, ab, o, w, u);
+      jacobian<IX, R, UNIT>(cr, q, yr, R(D) * jscale, ab, o, w, u);
     } else {
       jacobian<IX, R>(cr, q, yr, R(D), ab, o, w, u);
     }
@@ -178,13 +184,23 @@ __device__ __forceinline__ void eval_fj(const DigConst& c, const DigConstF* cf, 
     RS ys[NS];
 #pragma unroll
     for (int i = 0; i < NS; ++i) ys[i] = RS(y[i]);
+    Factors<RS> k;
+    factors<RS>(c, q, ys, ab, k);
     Rates<RS> o;
-    rates<RS, false>(c, q, ys, ab, o);
+    rates<RS, false>(c, q, ys, ab, k, o);
     RS fr[NS];
     balances<RS>(c, ys, RS(D), o, fr);
 #pragma unroll
     for (int i = 0; i < NS; ++i) f[i] = double(fr[i]);
   }
+}
+
+// g within about a factor of two of the positive S: on the bit patterns (an
+// FP64 compare occupies the FP64 pipe), whose high words are a
+// piecewise-linear log2; only which start a Newton takes hangs on it.
+__device__ __forceinline__ bool within_2x(double g, double S) {
+  const unsigned d = (unsigned)__double2hiint(g) - (unsigned)__double2hiint(S) + 0x00100000u;
+  return __double2hiint(g) > 0 && d < 0x00200000u;
 }
 
 // Newton guess for S_H at y + dy from the tangent dS_H/dy at y (Eq. 7
@@ -195,7 +211,7 @@ __device__ __forceinline__ double sh_guess(double SH0, const double* v, const do
                    v[2] * (y1[iS_pro] - y0[iS_pro]) + v[3] * (y1[iS_ac] - y0[iS_ac]) +
                    v[4] * (y1[iS_IC] - y0[iS_IC]) + v[5] * (y1[iS_IN] - y0[iS_IN]) +
                    v[6] * (y1[iS_cat] - y0[iS_cat]) + v[7] * (y1[iS_an] - y0[iS_an]);
-  return (g > 0.5 * SH0 && g < 2.0 * SH0) ? g : SH0;
+  return within_2x(g, SH0) ? g : SH0;
 }
 
 // W x = b with the factored W_d and the Sherman-Morrison vector q (the FP64
@@ -315,9 +331,33 @@ struct H2Split {
   }
 };
 
+// |d| as a float from its high word: truncated to 20 significand bits, below
+// the normal float range zero, above it (and for infinities and NaN) infinite.
+__device__ __forceinline__ float magf(double d) {
+  int m = (__double2hiint(d) & 0x7fffffff) - 0x38000000;
+  m = min(max(m, 0), 0x0ff00000);
+  return __uint_as_float((unsigned)m << 3);
+}
+
 // norm^(-1/3) of the step controller
 __device__ __forceinline__ float inv_cbrt(float x) { return rcbrtf(x); }
 __device__ __forceinline__ double inv_cbrt(double x) { return rcbrt(x); }
+
+// the eight states that enter Eq. 7
+__host__ __device__ constexpr bool in_eq7(int i) {
+  return i == iS_va || i == iS_bu || i == iS_pro || i == iS_ac || i == iS_IC || i == iS_IN ||
+         i == iS_cat || i == iS_an;
+}
+// S_h2 algebraic: the states that dS_h2/dy reaches (the S_h2 row of the
+// Jacobian and, through S_H, the states of Eq. 7), and those that the second
+// Sherman-Morrison vector p2 reaches (not the two ions, which only dilute,
+// nor S_h2 itself).  Products with the other entries are left out.
+__host__ __device__ constexpr bool h2_reads(int j) {
+  return j != iS_h2 && (sp::slot(iS_h2, j) >= 0 || in_eq7(j));
+}
+__host__ __device__ constexpr bool h2_moves(int i) {
+  return i != iS_h2 && i != iS_cat && i != iS_an;
+}
 
 template <int FORM, int BS, int MINB, bool WS>
 __global__ void __launch_bounds__(BS, MINB) integrate_kernel(StepArgs a) {
@@ -420,14 +460,14 @@ __global__ void __launch_bounds__(BS, MINB) integrate_kernel(StepArgs a) {
     }
     const double g = hh * kRB_d;
     AcidBase ab0;
-    // FP64: J_d and u come out scaled by -g, so W_d = I + (-g J_d) and
+    // FP64: W_d = I - g J_d comes out of the scatter, u scaled by -g:
     // q = W_d^-1 (g u) = -W_d^-1 (-g u)
     if constexpr (H2A)
-      eval_fj<R, RS, true, true, spa::Idx>(*c, cf, q, y, D, SHg, a.max_newton, cnt, F0,
+      eval_fj<R, RS, true, true, spa::Idx, spa::kNNZ>(*c, cf, q, y, D, SHg, a.max_newton, cnt, F0,
                                            H2Split<R, decltype(w)>{w, zh, p2}, qv, ko, ab0,
                                            R(-g), &SH2g);
     else
-      eval_fj<R, RS, !MIXED>(*c, cf, q, y, D, SHg, a.max_newton, cnt, F0, w, qv, ko, ab0,
+      eval_fj<R, RS, !MIXED, false, sp::Idx, sp::kNNZ>(*c, cf, q, y, D, SHg, a.max_newton, cnt, F0, w, qv, ko, ab0,
                              R(-g));
     const double SH0 = SHg;
     double vsh[8];
@@ -454,7 +494,7 @@ __global__ void __launch_bounds__(BS, MINB) integrate_kernel(StepArgs a) {
       for (int i = 0; i < NS; ++i) p2[i] = (sp::slot(i, iS_h2) >= 0 && i != iS_h2) ? -p2[i] : 0.0;
       qv[iS_h2] = R(0);
     }
-    LU::template form<R>(w, MIXED ? R(g) : R(-1));
+    if constexpr (MIXED) LU::template form<R>(w, R(g));
     const bool lu_ok = LU::template lu<R>(w);
     R inv_delta = R(0);
     // FP64: q and the Sherman-Morrison denominator here; mixed: in its loop
@@ -467,7 +507,8 @@ __global__ void __launch_bounds__(BS, MINB) integrate_kernel(StepArgs a) {
       rank1::update<double>(qv, vr, inv_delta, p2);
       double s2 = 0.0;
 #pragma unroll
-      for (int j = 0; j < NS; ++j) s2 += zh[j] * p2[j];
+      for (int j = 0; j < NS; ++j)
+        if (h2_reads(j)) s2 += zh[j] * p2[j];
       const double delta2 = 1.0 - s2;
       inv_delta2 = rcp<double>(delta2);
       piv_ok = piv_ok && isfinite(delta2) && delta2 != 0.0 &&
@@ -562,8 +603,9 @@ __global__ void __launch_bounds__(BS, MINB) integrate_kernel(StepArgs a) {
             // tangent guess of the Eq. 8 root at y1
             double g2 = SH20;
 #pragma unroll
-            for (int j = 0; j < NS; ++j) g2 += zh[j] * (y1[j] - y[j]);
-            SH2g = (g2 > 0.5 * SH20 && g2 < 2.0 * SH20) ? g2 : SH20;
+            for (int j = 0; j < NS; ++j)
+              if (h2_reads(j)) g2 += zh[j] * (y1[j] - y[j]);
+            SH2g = within_2x(g2, SH20) ? g2 : SH20;
             eval_f<RS, true>(*c, q, y1, D, SHg, a.max_newton, cnt, tmp, &SH2g);
           } else {
             eval_f<RS>(*c, q, y1, D, SHg, a.max_newton, cnt, tmp);
@@ -584,10 +626,12 @@ __global__ void __launch_bounds__(BS, MINB) integrate_kernel(StepArgs a) {
         if constexpr (H2A) {
           double s2 = 0.0;
 #pragma unroll
-          for (int j = 0; j < NS; ++j) s2 += zh[j] * xs[j];
+          for (int j = 0; j < NS; ++j)
+            if (h2_reads(j)) s2 += zh[j] * xs[j];
           s2 *= inv_delta2;
 #pragma unroll
-          for (int i = 0; i < NS; ++i) xs[i] += s2 * p2[i];
+          for (int i = 0; i < NS; ++i)
+            if (h2_moves(i)) xs[i] += s2 * p2[i];
         }
         if (st == 0) {
 #pragma unroll
@@ -604,19 +648,31 @@ __global__ void __launch_bounds__(BS, MINB) integrate_kernel(StepArgs a) {
       // Mixed forms: the combination, which cancels, in FP64, everything
       // after it in FP32 (the accept test needs a few digits only).
       if constexpr (!MIXED) {
-        // the largest ratio |e_i| / sc_i kept as the pair (en, sn), compared
-        // by cross products (sc_i > 0), so that one reciprocal suffices
-        double en = 0.0, sn = 1.0;
+        // The species with the largest ratio is found in FP32 (truncated
+        // high words, a few 1e-6 relative), its error and magnitude kept in
+        // FP64 and the norm formed from them: a near tie can pick a ratio
+        // 4e-6 below the largest.  Comparing 29 ratios in FP64 took five
+        // slots of the FP64 pipe per species.  Not finite -> the ratio is
+        // infinite and stays the largest.
+        double en = 0.0, ym = 0.0, at = 1.0;
+        float best = 0.0f;
+        const float rtol = cvt<float>(a.rtol);
 #pragma unroll
         for (int i = 0; i < NS; ++i) {
-          const double e = fabs(fma(-2.0, k2[i], k1[i]) + xs[i]);
-          const double sc = fma(a.rtol, fmax(fabs(y[i]), fabs(y1[i])), a.atol[i]);
-          if (!(e * sn <= en * sc)) {  // NaN propagates as in the ratio form
+          const double e = fma(-2.0, k2[i], k1[i]) + xs[i];
+          const double yi = mag64(y[i]) > mag64(y1[i]) ? y[i] : y1[i];
+          const float ef = magf(e), yf = magf(yi);
+          const float r = ef * rcp_approx(fmaf(rtol, yf, magf(a.atol[i])));
+          const bool inf = ef == INFINITY || yf == INFINITY;
+          if (inf ? best < INFINITY : r > best) {
+            best = inf ? INFINITY : r;
             en = e;
-            sn = sc;
+            ym = yi;
+            at = a.atol[i];
           }
         }
-        norm = en * rcp<double>(sn) * (hh * (1.0 / 6.0));
+        const double sn = fma(a.rtol, fabs(ym), at);
+        norm = fabs(en) * rcp<double>(sn) * (hh * (1.0 / 6.0));
       } else {
         float nf = 0.0f;
         const float rtol = cvt<float>(a.rtol);

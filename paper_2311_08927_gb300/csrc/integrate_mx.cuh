@@ -44,12 +44,6 @@ __device__ __forceinline__ int reread_i(int i) {
   return i;
 }
 
-// the eight states that enter Eq. 7
-__host__ __device__ constexpr bool in_eq7(int i) {
-  return i == iS_va || i == iS_bu || i == iS_pro || i == iS_ac || i == iS_IC || i == iS_IN ||
-         i == iS_cat || i == iS_an;
-}
-
 // binary64 -> float and float -> binary64 of the kernel (hardware conversions)
 __device__ __forceinline__ float f32(double d) { return float(d); }
 __device__ __forceinline__ double f64(float f) { return double(f); }
@@ -96,14 +90,16 @@ __device__ __forceinline__ float solve_h2_f32(const H2Bal<float>& e, float guess
 }
 
 // S_H (FP64 Newton at the FP64 state y) and S_h2 (FP32 Newton at the float
-// state ys, written into ys[iS_h2]) at one evaluation point.
+// state ys, written into ys[iS_h2]) at one evaluation point; k receives the
+// rate factors there.
 __device__ __forceinline__ void roots(const DigConst& c, const DigConstF& cf, const PartConst& q,
                                       const PartConstF& qf, const double* y, float* ys, float D,
                                       double& SHg, float& SH2g, int max_newton, Cnt& cnt,
-                                      AcidBase& ab) {
+                                      AcidBase& ab, Factors<float>& k) {
   newton(c, q, y, SHg, max_newton, cnt, ab);
+  factors<float>(cf, qf, ys, ab, k);
   H2Bal<float> e;
-  h2_coeffs<float>(cf, qf, ys, D, ab, e);
+  h2_coeffs<float>(cf, qf, ys, D, k, e);
   SH2g = solve_h2_f32(e, SH2g, cnt);
   ys[iS_h2] = SH2g;
 }
@@ -111,9 +107,9 @@ __device__ __forceinline__ void roots(const DigConst& c, const DigConstF& cf, co
 // FP32 rate vector at ys (roots already in ab and ys[iS_h2]); S_h2 rate 0.
 __device__ __forceinline__ void rates_f32(const DigConstF& cf, const PartConstF& qf,
                                           const float* ys, float D, const AcidBase& ab,
-                                          float* f) {
+                                          const Factors<float>& k, float* f) {
   Rates<float> o;
-  rates<float, false>(cf, qf, ys, ab, o);
+  rates<float, false>(cf, qf, ys, ab, k, o);
   balances<float>(cf, ys, D, o, f);
   f[iS_h2] = 0.0f;
 }
@@ -127,10 +123,12 @@ __device__ __forceinline__ void wsolve(W w, const float* qv,
   rank1::update<float>(qv, vr, inv_delta, x);
   float s2 = 0.0f;
 #pragma unroll
-  for (int j = 0; j < NS; ++j) s2 = fmaf(zh[j], x[j], s2);
+  for (int j = 0; j < NS; ++j)
+    if (h2_reads(j)) s2 = fmaf(zh[j], x[j], s2);
   s2 *= inv_delta2;
 #pragma unroll
-  for (int i = 0; i < NS; ++i) x[i] = fmaf(s2, p2[i], x[i]);
+  for (int i = 0; i < NS; ++i)
+    if (h2_moves(i)) x[i] = fmaf(s2, p2[i], x[i]);
 }
 
 // IDX: contexts with more than one digester, whose warps hold particles of
@@ -254,12 +252,13 @@ __global__ void __launch_bounds__(BS, MINB) integrate_mx_kernel(StepArgs a) {
     }
     // roots, rates, J_d and u at y (all FP32 but the Eq. 7 Newton)
     AcidBase ab0;
-    roots(dcn(), dcfn(), q, qf, y, ys, Df, SHg, SH2g, a.max_newton, cnt, ab0);
     {
+      Factors<float> k;
+      roots(dcn(), dcfn(), q, qf, y, ys, Df, SHg, SH2g, a.max_newton, cnt, ab0, k);
       // the rate partials are recomputed for each refinement residual
       // (from ys and ab0) rather than kept across the stages
       Rates<float> ko;
-      rates<float, true>(*cf, qf, ys, ab0, ko);
+      rates<float, true>(*cf, qf, ys, ab0, k, ko);
       balances<float>(*cf, ys, Df, ko, F0);
       F0[iS_h2] = 0.0f;
       jacobian<spa::Idx, float>(*cf, qf, ys, Df, ab0, ko,
@@ -301,7 +300,8 @@ __global__ void __launch_bounds__(BS, MINB) integrate_mx_kernel(StepArgs a) {
       rank1::update<float>(qv, vr, inv_delta, p2);
       float s2 = 0.0f;
 #pragma unroll
-      for (int j = 0; j < NS; ++j) s2 = fmaf(zh[j], p2[j], s2);
+      for (int j = 0; j < NS; ++j)
+        if (h2_reads(j)) s2 = fmaf(zh[j], p2[j], s2);
       const float delta2 = 1.0f - s2;
       inv_delta2 = rcp<float>(delta2);
       piv_ok = piv_ok && isfinite(delta2) && delta2 != 0.0f &&
@@ -366,13 +366,15 @@ __global__ void __launch_bounds__(BS, MINB) integrate_mx_kernel(StepArgs a) {
           {
             float g2 = SH20;
 #pragma unroll
-            for (int j = 0; j < NS; ++j) g2 = fmaf(zh[j], y1s[j] - ys[j], g2);
+            for (int j = 0; j < NS; ++j)
+              if (h2_reads(j)) g2 = fmaf(zh[j], y1s[j] - ys[j], g2);
             SH2g = (g2 > 0.5f * SH20 && g2 < 2.0f * SH20) ? g2 : SH20;
           }
           AcidBase ab;
-          roots(dcn(), dcfn(), q, qf, y1, y1s, Df, SHg, SH2g, a.max_newton, cnt, ab);
+          Factors<float> k;
+          roots(dcn(), dcfn(), q, qf, y1, y1s, Df, SHg, SH2g, a.max_newton, cnt, ab, k);
           float Fs[NS];
-          rates_f32(dcfn(), qf, y1s, Df, ab, Fs);
+          rates_f32(dcfn(), qf, y1s, Df, ab, k, Fs);
           if (st == 1) {
 #pragma unroll
             for (int i = 0; i < NS; ++i) {
@@ -401,7 +403,7 @@ __global__ void __launch_bounds__(BS, MINB) integrate_mx_kernel(StepArgs a) {
           DF zx(0.0f);
 #pragma unroll
           for (int j = 0; j < NS; ++j)
-            if (j != iS_h2) zx = zx + zh[j] * xp[j];
+            if (h2_reads(j)) zx = zx + zh[j] * xp[j];
           xp[iS_h2] = zx;
           DF sv(0.0f);
           {
@@ -411,7 +413,9 @@ __global__ void __launch_bounds__(BS, MINB) integrate_mx_kernel(StepArgs a) {
           }
           Rates<float> ko;
           const DigConstF& cfr = dcfn();
-          rates<float, true>(cfr, qf, ys, ab0, ko);
+          Factors<float> k;
+          factors<float>(cfr, qf, ys, ab0, k);
+          rates<float, true>(cfr, qf, ys, ab0, k, ko);
           jvp<float, DF, DigConstF, float>(cfr, ys, Df, ko, xp, sv, jx);
           jx[iS_h2] = DF(0.0f);
           float r[NS];

@@ -36,8 +36,10 @@ __host__ __device__ void eval_one(const EvalIn& in, EvalOut& out, bool split) {
   AcidBase ab;
   NewtonCounters nc{0, 0, 0};
   solve_SH(in.c, q, in.y, in.SH_guess, 50, ab, nc);
+  Factors<double> k;
+  factors<double>(in.c, q, in.y, ab, k);
   Rates<double> o;
-  rates<double, true>(in.c, q, in.y, ab, o);
+  rates<double, true>(in.c, q, in.y, ab, k, o);
   balances<double>(in.c, in.y, in.D, o, out.f);
   for (int i = 0; i < NS; ++i) out.u[i] = out.v[i] = 0.0;
   if (split) {

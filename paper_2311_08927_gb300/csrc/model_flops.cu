@@ -83,11 +83,12 @@ using namespace chad;
 // out[8] refinement update of one mixed solve (besides J x)
 // out[9] Sherman-Morrison set-up of one attempt (besides its solve)
 // out[10] Sherman-Morrison update of one solve
-// out[11] move of the acid-base reciprocals to a converged Newton root
-// out[12] scaling of the rate partials by -g (FP64 form's W formation)
+// out[11] once per Eq. 7 solve: the products of its balance, the third-order
+//         step and the move of the acid-base reciprocals to the root
+// out[12] 0 (the scaling of the rate partials by -g is part of out[1])
 // With n >= 18, the mixed form with S_h2 algebraic (kernel form 4) also:
 // out[13] J x from the FP32 rate partials in two-float arithmetic (FP32 flops)
-// out[14] coefficients of the Eq. 8 balance (h2_coeffs)
+// out[14] coefficients of the Eq. 8 balance (h2_coeffs, besides the shared factors)
 // out[15] one Eq. 8 Newton iteration (h2_eval + update)
 // out[16] FP32 work of one attempt besides rates, LU, solves, J x and Eq. 8
 // out[17] FP64 work of one attempt besides the Eq. 7 Newton iterations
@@ -117,20 +118,25 @@ extern "C" chad_status chad_flop_counts(int64_t* out, int n) {
   Fc y[NS], f[NS];
   for (int i = 0; i < NS; ++i) { yd[i] = 1.0; y[i] = Fc(1.0); }
   Rates<Fc> o;
+  Factors<Fc> k;
   g_ops = 0;
-  rates<Fc, false>(c, q, y, ab, o);
+  factors<Fc>(c, q, y, ab, k);
+  rates<Fc, false>(c, q, y, ab, k, o);
   balances<Fc>(c, y, Fc(0.1), o, f);
   out[0] = g_ops;
   static Fc w[sp::kNNZ];
   Fc u[NS];
   g_ops = 0;
-  rates<Fc, true>(c, q, y, ab, o);
+  factors<Fc>(c, q, y, ab, k);
+  rates<Fc, true>(c, q, y, ab, k, o);
   balances<Fc>(c, y, Fc(0.1), o, f);
   jacobian<sp::Idx, Fc>(c, q, y, Fc(0.1), ab, o, w, u);
   out[1] = g_ops;
   Fc r[6], rS, dE;
+  ChargeBalT<Fc> cb;
+  charge_bal<Fc>(c, q, yd, cb);
   g_ops = 0;
-  charge_E_t<Fc>(c, q, yd, Fc(1e-7), r, rS, dE);
+  charge_eval<Fc>(c, q, cb, Fc(1e-7), r, rS, dE);
   out[2] = g_ops;
   for (int s = 0; s < sp::kNNZ; ++s) w[s] = Fc(0.0);
   g_ops = 0;
@@ -161,11 +167,11 @@ extern "C" chad_status chad_flop_counts(int64_t* out, int n) {
   rank1::update<Fc>(u, v, inv_delta, b);
   out[10] = g_ops;
   g_ops = 0;
-  root_shift_t<Fc>(c, q, yd, Fc(1e-7), Fc(1e-16), r, rS, dE);
+  charge_bal<Fc>(c, q, yd, cb);
+  const Fc d = charge_step<Fc>(cb, Fc(q.K_w), rS, r, Fc(1e-16), Fc(1.0));
+  charge_move<Fc>(cb, Fc(q.K_w), Fc(1e-7), d, r, rS, dE);
   out[11] = g_ops;
-  g_ops = 0;
-  scale_partials<Fc>(o, Fc(-1e-4));
-  out[12] = g_ops;
+  out[12] = 0;
   // y + h/2 k1 (2/elt), F1 - k1 (1), k2 += k1 (1), y + h k2 (2), F2 - e32 (k2 - F1)
   // - 2 (k1 - F0) (5), h/6 (k1 - 2 k2 + k3) (4), atol + rtol max(..) (2), |e|/sc (1)
   out[7] = (int64_t)NS * 18;
@@ -183,7 +189,7 @@ extern "C" chad_status chad_flop_counts(int64_t* out, int n) {
     {
       H2Bal<Fc> e;
       g_ops = 0;
-      h2_coeffs<Fc>(c, q, y, Fc(0.1), ab, e);
+      h2_coeffs<Fc>(c, q, y, Fc(0.1), k, e);
       out[14] = g_ops;
       e.Kfa = e.Kc4 = e.Kpro = e.Kh2 = Fc(1.0);
       Fc dE;
@@ -215,7 +221,8 @@ extern "C" chad_status chad_flop_counts(int64_t* out, int n) {
     // out[18] rates with their partials alone (no balances, no Jacobian):
     // the form-4 refinement residual recomputes them at each stage
     g_ops = 0;
-    rates<Fc, true>(c, q, y, ab, o);
+    factors<Fc>(c, q, y, ab, k);
+    rates<Fc, true>(c, q, y, ab, k, o);
     out[18] = g_ops;
   }
   if (n >= 22) {

@@ -55,12 +55,14 @@ CHAD_HD bool setup(W w, R g, const R* v, R tau, R* q, R* inv_delta) {
   return isfinite(delta) && fabs(delta) >= tau * fmax(R(1), fabs(s)) && delta != R(0);
 }
 
-// z = W_d^-1 b (already solved) -> W^-1 b in place.
+// z = W_d^-1 b (already solved) -> W^-1 b in place.  S_cat and S_an only
+// dilute: q has no entry there.
 template <class R>
 CHAD_HD void update(const R* q, const R* v, R inv_delta, R* z) {
   const R s = vdot<R>(v, z) * inv_delta;
 #pragma unroll
-  for (int i = 0; i < NS; ++i) z[i] += s * q[i];
+  for (int i = 0; i < NS; ++i)
+    if (i != iS_cat && i != iS_an) z[i] += s * q[i];
 }
 
 }  // namespace rank1
