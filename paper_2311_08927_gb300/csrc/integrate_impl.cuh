@@ -101,14 +101,12 @@ __device__ __forceinline__ void newton_h2(const DigConst& c, const PartConst& q,
   cnt.failed |= nc.failed;
 }
 
-// f(y) in precision RS (Newton in FP64).  H2A: S_h2 algebraic (Eq. 8), its
-// root in *SH2g (guess in, root out) and a zero S_h2 rate.
+// f(y) in precision RS at the Eq. 7 root ab.  H2A: S_h2 algebraic (Eq. 8),
+// its root in *SH2g (guess in, root out) and a zero S_h2 rate.
 template <class RS, bool H2A = false>
 __device__ __forceinline__ void eval_f(const DigConst& c, const PartConst& q, const double* y,
-                                       double D, double& SHg, int max_newton, Cnt& cnt,
+                                       double D, const AcidBase& ab, int max_newton, Cnt& cnt,
                                        double* f, double* SH2g = nullptr) {
-  AcidBase ab;
-  newton(c, q, y, SHg, max_newton, cnt, ab);
   RS yr[NS];
 #pragma unroll
   for (int i = 0; i < NS; ++i) yr[i] = RS(y[i]);
@@ -127,8 +125,8 @@ __device__ __forceinline__ void eval_f(const DigConst& c, const PartConst& q, co
   if constexpr (H2A) f[iS_h2] = 0.0;
 }
 
-// f(y) in precision RS, J_d (sparse slots) and u = df/dS_H in precision R,
-// one Newton solve.  SCALE (FP64 form only, where R is RS): J_d and u come
+// f(y) in precision RS, J_d (sparse slots) and u = df/dS_H in precision R, at
+// the Eq. 7 root ab.  SCALE (FP64 form only, where R is RS): J_d and u come
 // out multiplied by jscale, and the slots below UNIT hold I + jscale J_d.
 // IX: the slot map of the Jacobian scatter (sp::Idx; with S_h2 algebraic
 // spa::Idx, with w an H2Split that takes S_h2's row and column apart).
@@ -151,11 +149,10 @@ struct DCSel<float> {
 template <class R, class RS, bool SCALE, bool H2A = false, class IX = sp::Idx, int UNIT = 0,
           class W>
 __device__ __forceinline__ void eval_fj(const DigConst& c, const DigConstF* cf, const PartConst& q,
-                                        const double* y, double D, double& SHg, int max_newton,
-                                        Cnt& cnt, double* f, W w, R* u, Rates<R>& o,
-                                        AcidBase& ab, R jscale, double* SH2g = nullptr) {
+                                        const double* y, double D, int max_newton, Cnt& cnt,
+                                        double* f, W w, R* u, Rates<R>& o, const AcidBase& ab,
+                                        R jscale, double* SH2g = nullptr) {
   const auto& cr = DCSel<R>::get(c, cf);
-  newton(c, q, y, SHg, max_newton, cnt, ab);
   {
     R yr[NS];
 #pragma unroll
@@ -275,7 +272,9 @@ __device__ __forceinline__ void stage_rhs(int st, const DigConst& c, const PartC
     for (int i = 0; i < NS; ++i) y1[i] = fma(hh, k2[i], y[i]);
   }
   SHg = sh_guess(SH0, vsh, y, y1);
-  eval_f<RS>(c, q, y1, D, SHg, max_newton, cnt, out);
+  AcidBase ab;
+  newton(c, q, y1, SHg, max_newton, cnt, ab);
+  eval_f<RS>(c, q, y1, D, ab, max_newton, cnt, out);
   if (st == 1) {
 #pragma unroll
     for (int i = 0; i < NS; ++i) {
@@ -412,11 +411,7 @@ __global__ void __launch_bounds__(BS, MINB) integrate_kernel(StepArgs a) {
         fresh = true;
       }
     }
-    // every thread of the block reaches this barrier once per iteration:
-    // the block's warps start each attempt together (shared instruction
-    // fetch); the loop ends when no thread of the block has a particle
-    if (!__syncthreads_or(p >= 0)) break;
-    if (p < 0) continue;
+    const bool act = p >= 0;
     if (fresh) {
       cnt = Cnt{0, 0, 0, 0, 0, 0, 0, 0};
       c = &a.dc[a.dig[p]];
@@ -451,7 +446,6 @@ __global__ void __launch_bounds__(BS, MINB) integrate_kernel(StepArgs a) {
     }
     // ------------------------------------------------ one step attempt
     bool done = false;
-    ++attempts;
     double hh = h;
     bool last = false;
     if (!fixed && hh >= (Tend - t) * (1.0 - 1e-12)) {
@@ -460,22 +454,41 @@ __global__ void __launch_bounds__(BS, MINB) integrate_kernel(StepArgs a) {
     }
     const double g = hh * kRB_d;
     AcidBase ab0;
+    double SH0 = 0.0, SH20 = 0.0, vsh[8];
+    R vr[8];
+    R inv_delta = R(0);
+    bool lu_ok = false, piv_ok = false;
+    if (act) {
+      ++attempts;
+      newton(*c, q, y, SHg, a.max_newton, cnt, ab0);
+    }
+    // Every thread of the block reaches this barrier once per attempt: the
+    // block's warps go through the straight-line code together and share the
+    // fetched instructions (the code is several times the instruction cache,
+    // and instruction fetch was the top stall where they did not).  It stands
+    // after the first Newton, where the states of a fresh particle have
+    // arrived from memory: ahead of the loads, the warps with a fresh lane
+    // fell behind the others by the loads' latency.  A second one follows
+    // each stage's Newton.  100,000 particles in the shared-headspace cylinder
+    // (FP64, S_h2 algebraic, 40 attempts per particle): 52.8 ms with the
+    // barrier ahead of the loads, 48.1 here, 45.2 with those of the stages.
+    // The loop ends when no thread of the block has a particle.
+    if (!__syncthreads_or(act)) break;
+    if (act) {
     // FP64: W_d = I - g J_d comes out of the scatter, u scaled by -g:
     // q = W_d^-1 (g u) = -W_d^-1 (-g u)
     if constexpr (H2A)
-      eval_fj<R, RS, true, true, spa::Idx, spa::kNNZ>(*c, cf, q, y, D, SHg, a.max_newton, cnt, F0,
+      eval_fj<R, RS, true, true, spa::Idx, spa::kNNZ>(*c, cf, q, y, D, a.max_newton, cnt, F0,
                                            H2Split<R, decltype(w)>{w, zh, p2}, qv, ko, ab0,
                                            R(-g), &SH2g);
     else
-      eval_fj<R, RS, !MIXED, false, sp::Idx, sp::kNNZ>(*c, cf, q, y, D, SHg, a.max_newton, cnt, F0, w, qv, ko, ab0,
-                             R(-g));
-    const double SH0 = SHg;
-    double vsh[8];
+      eval_fj<R, RS, !MIXED, false, sp::Idx, sp::kNNZ>(*c, cf, q, y, D, a.max_newton, cnt, F0, w, qv, ko,
+                                                       ab0, R(-g));
+    SH0 = SHg;
+    SH20 = SH2g;
     sh_tangent(*c, q, ab0, vsh);
-    R vr[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) vr[k] = R(vsh[k]);
-    const double SH20 = SH2g;
     if constexpr (H2A) {
       // The S_h2 row of -g J_d (delivered into zh by the scatter) gives
       // dS_h2/dy = -(J_h2,j + u_h2 v_j) / J_h2,h2 (the scale cancels); its
@@ -495,11 +508,10 @@ __global__ void __launch_bounds__(BS, MINB) integrate_kernel(StepArgs a) {
       qv[iS_h2] = R(0);
     }
     if constexpr (MIXED) LU::template form<R>(w, R(g));
-    const bool lu_ok = LU::template lu<R>(w);
-    R inv_delta = R(0);
+    lu_ok = LU::template lu<R>(w);
     // FP64: q and the Sherman-Morrison denominator here; mixed: in its loop
     const bool sm_ok = MIXED || rank1::setup<R, LU>(w, R(-1), vr, R(kPivTau), qv, &inv_delta);
-    bool piv_ok = lu_ok && sm_ok;
+    piv_ok = lu_ok && sm_ok;
     if constexpr (H2A) {
       // p2 = W_1^-1 (g w) with W_1 = W_d - g u v^T (first Sherman-Morrison
       // level), then the second level's denominator 1 - zh^T p2
@@ -514,10 +526,11 @@ __global__ void __launch_bounds__(BS, MINB) integrate_kernel(StepArgs a) {
       piv_ok = piv_ok && isfinite(delta2) && delta2 != 0.0 &&
                fabs(delta2) >= kPivTau * fmax(1.0, fabs(s2));
     }
+    }
     // error norm and controller: FP64 in the FP64 forms, FP32 in the mixed ones
     using NR = typename std::conditional<MIXED, float, double>::type;
     NR norm = NR(INFINITY);
-    if (!MIXED && !piv_ok) cnt.pivot++;
+    if (!MIXED && act && !piv_ok) cnt.pivot++;
     double xs[NS];
     if constexpr (MIXED) {
       // Mixed: one loop over q (st = -1) and the stages, and within a stage
@@ -527,7 +540,7 @@ __global__ void __launch_bounds__(BS, MINB) integrate_kernel(StepArgs a) {
       // larger than the instruction cache).  The FP32<->FP64 conversions use
       // the hardware instructions: ~120 per stage, which as integer
       // sequences cost more issue slots than they free on the FP64 pipe.
-      if (lu_ok || fixed) {
+      if (act && (lu_ok || fixed)) {
         R t[NS];
 #pragma unroll 1
         for (int st = -1; st < 3; ++st) {
@@ -574,8 +587,8 @@ __global__ void __launch_bounds__(BS, MINB) integrate_kernel(StepArgs a) {
           }
         }
       }
-      if (!piv_ok) cnt.pivot++;
-    } else if (piv_ok || fixed) {
+      if (act && !piv_ok) cnt.pivot++;
+    } else {
       // The three stages share one factorisation.  They run as a loop that
       // is not unrolled, so the kernel holds a single copy of the solve and
       // of the rate evaluation (the straight-line code is large):
@@ -583,12 +596,11 @@ __global__ void __launch_bounds__(BS, MINB) integrate_kernel(StepArgs a) {
       //   stage 1: F1 = f(y + h/2 k1), x = W^-1 (F1 - k1) -> k2 = x + k1
       //   stage 2: F2 = f(y + h k2), x = W^-1 (F2 - e32 (k2 - F1) - 2 (k1 - F0))
       //            -> k3 = x (left in xs), y1 = y + h k2
+      const bool go = act && (piv_ok || fixed);
 #pragma unroll 1
       for (int st = 0; st < 3; ++st) {
-        if (st == 0) {
-#pragma unroll
-          for (int i = 0; i < NS; ++i) tmp[i] = F0[i];
-        } else {
+        AcidBase ab;
+        if (go && st > 0) {
           // separate loops per stage: a per-element select would evaluate both sides
           if (st == 1) {
             const double h2 = 0.5 * hh;
@@ -599,6 +611,14 @@ __global__ void __launch_bounds__(BS, MINB) integrate_kernel(StepArgs a) {
             for (int i = 0; i < NS; ++i) y1[i] = fma(hh, k2[i], y[i]);
           }
           SHg = sh_guess(SH0, vsh, y, y1);
+          newton(*c, q, y1, SHg, a.max_newton, cnt, ab);
+        }
+        __syncthreads();  // the warps leave the Newton together (as above)
+        if (!go) continue;
+        if (st == 0) {
+#pragma unroll
+          for (int i = 0; i < NS; ++i) tmp[i] = F0[i];
+        } else {
           if constexpr (H2A) {
             // tangent guess of the Eq. 8 root at y1
             double g2 = SH20;
@@ -606,9 +626,9 @@ __global__ void __launch_bounds__(BS, MINB) integrate_kernel(StepArgs a) {
             for (int j = 0; j < NS; ++j)
               if (h2_reads(j)) g2 += zh[j] * (y1[j] - y[j]);
             SH2g = within_2x(g2, SH20) ? g2 : SH20;
-            eval_f<RS, true>(*c, q, y1, D, SHg, a.max_newton, cnt, tmp, &SH2g);
+            eval_f<RS, true>(*c, q, y1, D, ab, a.max_newton, cnt, tmp, &SH2g);
           } else {
-            eval_f<RS>(*c, q, y1, D, SHg, a.max_newton, cnt, tmp);
+            eval_f<RS>(*c, q, y1, D, ab, a.max_newton, cnt, tmp);
           }
           if (st == 1) {
 #pragma unroll
@@ -642,6 +662,7 @@ __global__ void __launch_bounds__(BS, MINB) integrate_kernel(StepArgs a) {
         }
       }
     }
+    if (!act) continue;
     if (piv_ok || fixed) {
       // scaled error norm max_i |h/6 (k1 - 2 k2 + k3)_i| / (atol_i + rtol
       // max(|y_i|, |y1_i|)).  FP64 forms: all of it in FP64, as the oracle.
