@@ -92,8 +92,7 @@ struct chad_ctx {
   int* d_order_cnt = nullptr;  // [2 * kOrderBuckets] bucket counts and cursors
   unsigned long long* d_misc = nullptr;  // [2]: load check flag, failed-particle count
   unsigned long long* d_interval = nullptr;  // global interval index (noise counter)
-  int variant[5] = {kDefaultVariant, kDefaultVariant, kDefaultVariant, kDefaultVariant,
-                    kDefaultVariant};
+  int variant[5] = {0, 0, 0, 0, 0};  // per kernel form; by size until asked otherwise
   double flow_dt = -1.0;        // interval length the device flow constants hold
   // CUDA graph of one interval (captured on first use, replayed per interval)
   cudaGraphExec_t gexec = nullptr;
@@ -271,6 +270,12 @@ chad_status chad_create(const chad_config* cfg, chad_ctx** out) {
   c->diff_D.assign(c->n_dig, 0.0);
   c->diff_h.assign(c->n_dig, 0.0);
   c->loaded.assign(c->n_dig, 0);
+  {
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    for (int f = 0; f < 5; ++f) c->variant[f] = default_variant(f, c->N, sms);
+  }
   for (int d = 0; d < c->n_dig; ++d) {
     const char* why = "";
     const double Du = cfg->D_uniform ? cfg->D_uniform[d] : 0.0;

@@ -22,7 +22,7 @@ cudaError_t launch_integrate(const StepArgs& a, int precision, int variant, cuda
                                             CHAD_ROW(4)};
 #undef CHAD_ROW
   if (a.n <= 0) return cudaSuccess;
-  if (variant < 0 || variant >= kNumVariants) variant = kDefaultVariant;
+  if (variant < 0 || variant >= kNumVariants) variant = 0;
   if (precision < 0 || precision > 4) precision = 0;
   return table[precision][variant](a, s);
 }

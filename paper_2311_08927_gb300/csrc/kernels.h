@@ -72,13 +72,13 @@ struct HeadspaceArgs {
 };
 
 // Integrator kernel variants, chosen per context and kernel form by the
-// autotuner: threads per block, minimum resident blocks per SM (which sets
-// the register budget, 65536 / (threads x blocks) up to 255) and where the
-// factored matrix W_d lives (0: per-thread arrays, i.e. registers spilling to
-// local memory; 1: the thread's column of a shared-memory tile, 128 threads
-// for the float forms, 64 for the FP64 forms, 2 blocks per SM).
+// population's size (default_variant) or the autotuner: threads per block,
+// minimum resident blocks per SM (which sets the register budget, 65536 /
+// (threads x blocks) up to 255) and where the factored matrix W_d lives (0:
+// per-thread arrays, i.e. registers spilling to local memory; 1: the thread's
+// column of a shared-memory tile, 256 threads for form 4, 128 for forms 1
+// and 2, 64 for the FP64 forms).
 constexpr int kNumVariants = 7;
-constexpr int kDefaultVariant = 0;
 struct KernelVariant {
   int threads, min_blocks, w_shared;
 };
@@ -90,7 +90,21 @@ constexpr KernelVariant kernel_variant(int form, int v) {
          : v == 3 ? KernelVariant{64, 4, 0}
          : v == 4 ? KernelVariant{256, 1, 0}
          : v == 5 ? KernelVariant{32, 8, 0}
-                  : KernelVariant{(form == 0 || form == 3) ? 64 : 128, 2, 1};
+         : form == 4 ? KernelVariant{256, 1, 1}
+                     : KernelVariant{(form == 0 || form == 3) ? 64 : 128, 2, 1};
+}
+// The variant of a context that asked for none.  Few particles: small blocks
+// spread them over the SMs, so that a warp has its sub-partition's FP64 pipe
+// (one warp instruction per 64 cycles) to itself: 1,000 particles FP64 with
+// S_h2 algebraic 3.23 ms with 128-thread blocks, 2.93 with 32; 20,000
+// particles FP64 11.8 ms against 10.7 with 64.  From about one 160-particle
+// share per SM on, large blocks, whose warps share the fetched code: 45,000
+// particles FP64 15.2 ms with 128 threads, 17.1 with 64.  There form 4 takes
+// one block of eight warps per SM with W_d in shared memory: 64 digesters
+// with 400,000 particles 115.9 ms (128 threads, W_d in registers) against
+// 83.1, 1M particles with slugs 34.0 against 27.1.
+constexpr int default_variant(int form, int64_t n, int sms) {
+  return n <= (int64_t)64 * sms ? 5 : n <= (int64_t)160 * sms ? 3 : form == 4 ? 6 : 0;
 }
 cudaError_t launch_integrate(const StepArgs& a, int precision, int variant, cudaStream_t s);
 cudaError_t launch_advect(const AdvectArgs& a, cudaStream_t s);

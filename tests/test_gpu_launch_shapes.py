@@ -1,0 +1,45 @@
+"""The launch shape that a context takes by its particle count (no autotuner,
+no explicit variant) gives the results of an explicit shape, around the counts
+where the rule changes and at the ends of the range."""
+import numpy as np
+import pytest
+
+from paper_2311_08927_gb300 import chad as CH
+from paper_2311_08927_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def sms():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2311_08927_gb300 import build
+    build.build()
+    return torch.cuda.get_device_properties(0).multi_processor_count
+
+
+def _run(pop, variant, **kw):
+    sim = CH.Simulator(pop, fixed_substeps=2, **kw)
+    if variant is not None:
+        CH.chad_set_kernel_variant(sim.ctx, variant)
+    sim.load()
+    sim.step(60.0, 1)
+    out = sim.read()
+    sim.close()
+    return out
+
+
+# FP64: two fixed steps of the same operations, whose contraction may differ
+# between the instances: some 1e3 roundings of 1.1e-16.  Mixed: FP32 stage
+# vectors (6e-8) times the relative change of a state over the interval (< 1).
+@pytest.mark.parametrize("kw,tol", [(dict(precision=CH.PREC_FP64, h2_algebraic=True), 1e-12),
+                                    (dict(precision=CH.PREC_MIXED, h2_algebraic=True), 1e-6)])
+@pytest.mark.parametrize("per_sm,extra", [(0, 1), (64, 0), (64, 1), (160, 0), (160, 1), (300, 7)])
+def test_default_shape_equals_an_explicit_one(sms, kw, tol, per_sm, extra):
+    pop = I.config_population(3, n=per_sm * sms + extra)
+    a, b = _run(pop, None, **kw), _run(pop, 0, **kw)
+    floor = 1e-12 * np.abs(b["y"]).max(axis=1, keepdims=True) + 1e-300
+    assert (np.abs(a["y"] - b["y"]) / np.maximum(np.abs(b["y"]), floor)).max() <= tol
+    assert np.array_equal(a["status"], b["status"])
