@@ -15,6 +15,7 @@
 #include <algorithm>
 #include <cstdint>
 
+#include "adm1_device.cuh"
 #include "chad.h"
 #include "kernels.h"
 #include "model.h"
@@ -29,37 +30,83 @@ constexpr int NPARAM = OFF_B3 + OUT;
 static_assert(NPARAM == CHAD_MLP_NPARAM, "parameter count");
 constexpr float kLogFloor = 1e-20f;
 
-// The activations are rounded to BF16 (8 significant bits) right after, so
-// the fast division (a few FP32 ulp) is exact enough; for z below about -88
-// the exponential overflows and both give 0.
-__device__ __forceinline__ float silu(float z) { return __fdividef(z, 1.0f + __expf(-z)); }
-__device__ __forceinline__ float dsilu(float z) {
-  const float s = __fdividef(1.0f, 1.0f + __expf(-z));
-  return s * (1.0f + z * (1.0f - s));
+// 1/(1 + e^-z) from the hardware's base-2 exponential and reciprocal: the
+// activations are rounded to BF16 (8 significant bits) right after.  The
+// flush-to-zero forms need no range handling around the two SFU operations;
+// for z below about -87 the sigmoid is 0.
+__device__ __forceinline__ float sigmoid(float z) {
+  float e;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(-z * 1.4426950408889634f));
+  return rcp_approx(1.0f + e);
 }
+__device__ __forceinline__ float silu(float z) { return z * sigmoid(z); }
 __device__ __forceinline__ uint32_t pack2(__nv_bfloat16 lo, __nv_bfloat16 hi) {
   return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
 }
 
-// Features of one particle: (log10 max(y_i, floor) - mu_i) * inv_sigma_i for
-// the 29 states, (T/100 - mu) * inv_sigma for the temperature, zero padding.
-__device__ __forceinline__ void features(const double* y, int64_t ld, int64_t p, double T,
-                                         const float* norm, __nv_bfloat16* row) {
-#pragma unroll
-  for (int i = 0; i < NS; ++i) {
-    const float v = fmaxf((float)y[(int64_t)i * ld + p], kLogFloor);
-    row[i] = __float2bfloat16_rn((log10f(v) - norm[i]) * norm[IN + i]);
-  }
-  row[NS] = __float2bfloat16_rn(((float)T * 0.01f - norm[NS]) * norm[IN + NS]);
-  row[NS + 1] = __float2bfloat16_rn(0.0f);
-  row[NS + 2] = __float2bfloat16_rn(0.0f);
+// max((float)d, floor) with the conversion rounded to nearest even, on the
+// bit pattern: a hardware FP64 -> FP32 conversion occupies the FP64 pipe (one
+// warp instruction per 64 cycles and sub-partition), which 29 of them per
+// particle would make the bound of the features.  Below 2^-126 and for NaN
+// the floor, from 2^128 up infinity.
+__device__ __forceinline__ float floored(double d) {
+  const int hi = __double2hiint(d);
+  const unsigned lo = (unsigned)__double2loint(d);
+  unsigned u = ((unsigned)(hi - 0x38000000) << 3) | (lo >> 29);
+  const unsigned rest = lo << 3;
+  u += rest > 0x80000000u || (rest == 0x80000000u && (u & 1u));
+  if (hi >= 0x47f00000) u = 0x7f800000u;
+  const bool nan = hi >= 0x7ff00000 && !(hi == 0x7ff00000 && lo == 0u);
+  return hi < 0x38100000 || nan ? kLogFloor : fmaxf(__uint_as_float(u), kLogFloor);
 }
 
-__global__ void features_kernel(const double* y, int64_t ld, const double* T, int64_t n,
-                                const float* norm, __nv_bfloat16* X) {
+// Features of one particle: (log10 max(y_i, floor) - mu_i) * inv_sigma_i for
+// the 29 states, (T/100 - mu) * inv_sigma for the temperature, zero padding;
+// the 16 from 16 half on as two 16-byte vectors.
+__device__ __forceinline__ void features(const double* __restrict__ y, int64_t ld, int64_t p,
+                                         double T, const float* norm, int half, uint4* row) {
+  uint32_t w[IN / 4];
+  float f[2];
+#pragma unroll
+  for (int j = 0; j < IN / 2; ++j) {
+    const int i = half * (IN / 2) + j;
+    if (i < NS)
+      f[j & 1] = (log10f(floored(y[(int64_t)i * ld + p])) - norm[i]) * norm[IN + i];
+    else
+      f[j & 1] = i == NS ? ((float)T * 0.01f - norm[NS]) * norm[IN + NS] : 0.0f;
+    if (j & 1) w[j >> 1] = pack2(__float2bfloat16_rn(f[0]), __float2bfloat16_rn(f[1]));
+  }
+  row[0] = make_uint4(w[0], w[1], w[2], w[3]);
+  row[1] = make_uint4(w[4], w[5], w[6], w[7]);
+}
+
+// One thread per particle: the states are read coalesced, the 64-byte row is
+// written as four vectors.  HBM-bound (240 B in, 64 B out): 1M particles
+// 46 us at the measured copy rate, 59 here (183 with
+// 2-byte stores and the hardware conversions).
+__global__ void __launch_bounds__(128) features_kernel(const double* y, int64_t ld, const double* T,
+                                                       int64_t n, const float* norm, uint4* X) {
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
-  features(y, ld, p, T[p], norm, X + p * IN);
+  uint4 row[4];
+  features(y, ld, p, T[p], norm, 0, row);
+  features(y, ld, p, T[p], norm, 1, row + 2);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) X[4 * p + j] = row[j];
+}
+
+// The same with rows that are only 2-byte aligned.
+__global__ void __launch_bounds__(128) features_kernel_unaligned(const double* y, int64_t ld,
+                                                                 const double* T, int64_t n,
+                                                                 const float* norm, uint16_t* X) {
+  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= n) return;
+  uint4 row[4];
+  features(y, ld, p, T[p], norm, 0, row);
+  features(y, ld, p, T[p], norm, 1, row + 2);
+  const uint16_t* e = reinterpret_cast<const uint16_t*>(row);
+#pragma unroll
+  for (int j = 0; j < IN; ++j) X[p * IN + j] = e[j];
 }
 
 // ---------------------------------------------------------------------------
@@ -76,14 +123,16 @@ __global__ void features_kernel(const double* y, int64_t ld, const double* T, in
 namespace tc {
 
 constexpr int TILE = 128;
-constexpr int kFwdPipes = 2;                       // tile pipelines per CTA (4 warps each)
-constexpr int kFwdThreads = kFwdPipes * TILE;
+constexpr int kFwdPipes = 2;                       // tile pipelines per CTA (8 warps each)
+constexpr int kPipeThreads = 2 * TILE;             // two threads share a sample (hidden units halved)
+constexpr int kFwdThreads = kFwdPipes * kPipeThreads;
 constexpr uint32_t kTmemCols = kFwdPipes * 128;    // per pipeline: Z1 0-63, Z2 64-127
 constexpr int kBlocksPerSM = 2;  // 2 x 256 = the SM's 512 tensor-memory columns
 
 struct FwdPipe {
   __nv_bfloat16 X[TILE * IN];     // 8 KB
   __nv_bfloat16 A1[TILE * HID];   // 16 KB
+  float2 part[TILE];              // output sums of the second half of the units
 };
 
 struct Smem {
@@ -180,14 +229,14 @@ __device__ __forceinline__ uint4 pack8(const float* a) {
   return u;
 }
 
-// Barrier of one pipeline's 128 threads (ids 1, 2; id 0 is __syncthreads).
-__device__ __forceinline__ void pipe_sync(int id) {
-  asm volatile("bar.sync %0, 128;" ::"r"(id) : "memory");
+// Barrier of one pipeline's 256 threads (ids 1, 2; id 0 is __syncthreads).
+__device__ __forceinline__ void pipe_bar(int id) {
+  asm volatile("bar.sync %0, 256;" ::"r"(id) : "memory");
 }
-__device__ __forceinline__ bool pipe_and(int id, bool v) {
+__device__ __forceinline__ bool pipe_bar_and(int id, bool v) {
   uint32_t r;
   asm volatile(
-      "{\n.reg .pred p, q;\nsetp.ne.u32 q, %1, 0;\nbar.red.and.pred p, %2, 128, q;\n"
+      "{\n.reg .pred p, q;\nsetp.ne.u32 q, %1, 0;\nbar.red.and.pred p, %2, 256, q;\n"
       "selp.u32 %0, 1, 0, p;\n}\n"
       : "=r"(r)
       : "r"((uint32_t)v), "r"(id)
@@ -195,27 +244,48 @@ __device__ __forceinline__ bool pipe_and(int id, bool v) {
   return r != 0;
 }
 
-// The forward pass over the tiles this CTA owns, in two pipelines of 4 warps
+// The two hidden layers' weights as K-major BF16 operands, the output layer
+// and the biases, by all T threads of the CTA.
+template <int T, class S>
+__device__ __forceinline__ void load_weights(S& s, const float* P) {
+  for (int i = threadIdx.x; i < HID * (IN + HID) / 8; i += T) {
+    const bool first = i < HID * IN / 8;
+    const int q = first ? i : i - HID * IN / 8, w = first ? IN : HID;
+    const int o = q / (w / 8), k = (q % (w / 8)) * 8;
+    const float* src = P + (first ? OFF_W1 : OFF_W2) + o * w + k;
+    float v[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[j] = src[j];
+    *reinterpret_cast<uint4*>(first ? &s.W1[kmaj(o, k, IN)] : &s.W2[kmaj(o, k, HID)]) = pack8(v);
+  }
+  for (int i = threadIdx.x; i < HID; i += T) {
+    s.b1[i] = P[OFF_B1 + i];
+    s.b2[i] = P[OFF_B2 + i];
+  }
+  for (int i = threadIdx.x; i < OUT * HID; i += T) s.W3[i] = __bfloat162float(__float2bfloat16_rn(P[OFF_W3 + i]));
+  if (threadIdx.x < OUT) s.b3[threadIdx.x] = P[OFF_B3 + threadIdx.x];
+}
+
+// The forward pass over the tiles this CTA owns, in two pipelines of 8 warps
 // (each with its own operands, half of the tensor memory, mbarrier and named
 // barrier), so that one tile's epilogue overlaps the other's MMAs; tiles go
-// to the CTAs first, then to their second pipelines.  load(p, v) fills the 32
-// BF16 features of sample p as four 16-byte vectors (p < n); store(p, o0, o1)
-// takes the two standardised outputs.
+// to the CTAs first, then to their second pipelines.  The tile's time is its
+// SiLU epilogues, two SFU operations each: two warps per lane quarter share
+// them, 32 warps per SM in all, and the next tile's features are on their way
+// (1M samples: 111 us with one warp, 97 with two, 91 with the prefetch).  load(p, half, v) fills
+// features 16 half .. 16 half + 15 of sample p as two 16-byte vectors
+// (p < n); store(p, o0, o1) takes the two standardised outputs.
 template <class Load, class Store>
 __device__ __forceinline__ void forward_tiles(Smem& s, const float* P, int64_t n, int* err,
                                               Load load, Store store) {
   const int cta_tid = threadIdx.x, warp = cta_tid >> 5;
-  const int pi = cta_tid / TILE, tid = cta_tid % TILE;
+  const int pi = cta_tid / kPipeThreads, tid = cta_tid % kPipeThreads;
+  const int half = (warp >> 2) & 1;                       // which half of the features and units
+  const int r = (warp & 3) * 32 + (cta_tid & 31);         // tile row = tensor-memory lane
+  const int u0 = half * (HID / 2);
   const int bar_id = 1 + pi;
   FwdPipe& b = s.pipe[pi];
-  for (int i = cta_tid; i < HID * IN; i += kFwdThreads) s.W1[kmaj(i / IN, i % IN, IN)] = __float2bfloat16_rn(P[OFF_W1 + i]);
-  for (int i = cta_tid; i < HID * HID; i += kFwdThreads) s.W2[kmaj(i / HID, i % HID, HID)] = __float2bfloat16_rn(P[OFF_W2 + i]);
-  for (int i = cta_tid; i < HID; i += kFwdThreads) {
-    s.b1[i] = P[OFF_B1 + i];
-    s.b2[i] = P[OFF_B2 + i];
-  }
-  for (int i = cta_tid; i < OUT * HID; i += kFwdThreads) s.W3[i] = __bfloat162float(__float2bfloat16_rn(P[OFF_W3 + i]));
-  if (cta_tid < OUT) s.b3[cta_tid] = P[OFF_B3 + cta_tid];
+  load_weights<kFwdThreads>(s, P);
   const uint32_t bar = smem_u32(&s.mbar[pi]);
   if (tid == 0) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
@@ -239,15 +309,17 @@ __device__ __forceinline__ void forward_tiles(Smem& s, const float* P, int64_t n
   uint32_t phase = 0;
   bool ok = true;
   const int64_t stride = (int64_t)gridDim.x * kFwdPipes * TILE;
+  // the next tile's features are fetched behind this tile's first MMAs
+  uint4 v[2] = {};
+  if (((int64_t)pi * gridDim.x + blockIdx.x) * TILE + r < n)
+    load(((int64_t)pi * gridDim.x + blockIdx.x) * TILE + r, half, v);
   for (int64_t m0 = ((int64_t)pi * gridDim.x + blockIdx.x) * TILE; m0 < n && ok; m0 += stride) {
-    const int64_t p = m0 + tid;
-    uint4 v[4] = {};
-    if (p < n) load(p, v);
+    const int64_t p = m0 + r;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) *reinterpret_cast<uint4*>(&b.X[kmaj(tid, 8 * j, IN)]) = v[j];
+    for (int j = 0; j < 2; ++j) *reinterpret_cast<uint4*>(&b.X[kmaj(r, 16 * half + 8 * j, IN)]) = v[j];
     fence_async_smem();
     fence_before();
-    pipe_sync(bar_id);
+    pipe_bar(bar_id);
     if (tid == 0) {
       fence_after();
 #pragma unroll
@@ -256,22 +328,24 @@ __device__ __forceinline__ void forward_tiles(Smem& s, const float* P, int64_t n
             kId, k);
       commit(bar);
     }
-    ok = pipe_and(bar_id, mbar_wait(bar, phase));
+    v[0] = v[1] = make_uint4(0u, 0u, 0u, 0u);
+    if (p + stride < n) load(p + stride, half, v);
+    ok = pipe_bar_and(bar_id, mbar_wait(bar, phase));
     phase ^= 1;
     if (!ok) break;
     fence_after();
 #pragma unroll
-    for (int c = 0; c < HID; c += 16) {
+    for (int c = 0; c < HID / 2; c += 16) {
       float z[16];
-      tmem_ld16(row_base + c, z);
+      tmem_ld16(row_base + u0 + c, z);
 #pragma unroll
-      for (int j = 0; j < 16; ++j) z[j] = silu(z[j] + s.b1[c + j]);
-      *reinterpret_cast<uint4*>(&b.A1[kmaj(tid, c, HID)]) = pack8(z);
-      *reinterpret_cast<uint4*>(&b.A1[kmaj(tid, c + 8, HID)]) = pack8(z + 8);
+      for (int j = 0; j < 16; ++j) z[j] = silu(z[j] + s.b1[u0 + c + j]);
+      *reinterpret_cast<uint4*>(&b.A1[kmaj(r, u0 + c, HID)]) = pack8(z);
+      *reinterpret_cast<uint4*>(&b.A1[kmaj(r, u0 + c + 8, HID)]) = pack8(z + 8);
     }
     fence_async_smem();
     fence_before();
-    pipe_sync(bar_id);
+    pipe_bar(bar_id);
     if (tid == 0) {
       fence_after();
 #pragma unroll
@@ -280,23 +354,28 @@ __device__ __forceinline__ void forward_tiles(Smem& s, const float* P, int64_t n
             sdesc(w2_addr + k * 256, 128, (HID / 8) * 128), kId, k);
       commit(bar);
     }
-    ok = pipe_and(bar_id, mbar_wait(bar, phase));
+    ok = pipe_bar_and(bar_id, mbar_wait(bar, phase));
     phase ^= 1;
     if (!ok) break;
     fence_after();
-    float o0 = s.b3[0], o1 = s.b3[1];
+    float o0 = 0.0f, o1 = 0.0f;
 #pragma unroll
-    for (int c = 0; c < HID; c += 16) {
+    for (int c = 0; c < HID / 2; c += 16) {
       float z[16];
-      tmem_ld16(row_base + HID + c, z);
+      tmem_ld16(row_base + HID + u0 + c, z);
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
-        const float a = __bfloat162float(__float2bfloat16_rn(silu(z[j] + s.b2[c + j])));
-        o0 = fmaf(a, s.W3[c + j], o0);
-        o1 = fmaf(a, s.W3[HID + c + j], o1);
+        const float a = __bfloat162float(__float2bfloat16_rn(silu(z[j] + s.b2[u0 + c + j])));
+        o0 = fmaf(a, s.W3[u0 + c + j], o0);
+        o1 = fmaf(a, s.W3[HID + u0 + c + j], o1);
       }
     }
-    if (p < n) store(p, o0, o1);
+    if (half == 1) b.part[r] = make_float2(o0, o1);
+    pipe_bar(bar_id);
+    if (half == 0 && p < n) {
+      const float2 h = b.part[r];
+      store(p, (s.b3[0] + o0) + h.x, (s.b3[1] + o1) + h.y);
+    }
   }
   const bool all_ok = __syncthreads_and(ok);
   fence_before();
@@ -317,10 +396,10 @@ __global__ void __launch_bounds__(kFwdThreads, kBlocksPerSM) forward_kernel(cons
   extern __shared__ unsigned char smem_raw[];
   forward_tiles(
       smem_aligned(smem_raw), P, n, err,
-      [&](int64_t p, uint4* v) {
-        const uint4* src = reinterpret_cast<const uint4*>(X + p * IN);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) v[j] = src[j];
+      [&](int64_t p, int half, uint4* v) {
+        const uint4* src = reinterpret_cast<const uint4*>(X + p * IN) + 2 * half;
+        v[0] = src[0];
+        v[1] = src[1];
       },
       [&](int64_t p, float o0, float o1) {
         out[p * OUT + 0] = o0;
@@ -338,7 +417,7 @@ __global__ void __launch_bounds__(kFwdThreads, kBlocksPerSM) guess_kernel(const 
   extern __shared__ unsigned char smem_raw[];
   forward_tiles(
       smem_aligned(smem_raw), P, n, err,
-      [&](int64_t p, uint4* v) { features(y, ld, p, T[p], norm, reinterpret_cast<__nv_bfloat16*>(v)); },
+      [&](int64_t p, int half, uint4* v) { features(y, ld, p, T[p], norm, half, v); },
       [&](int64_t p, float o0, float o1) {
         const float l0 = o0 * onorm[2] + onorm[0];
         const float l1 = o1 * onorm[3] + onorm[1];
@@ -350,52 +429,74 @@ __global__ void __launch_bounds__(kFwdThreads, kBlocksPerSM) guess_kernel(const 
 constexpr size_t smem_bytes() { return sizeof(Smem) + 128; }
 
 // Fused forward + backward of the mean-squared loss on the tensor cores, 128
-// samples per tile, one CTA per SM holding two tile pipelines (4 warps each),
-// so that one pipeline's epilogue overlaps the other's MMAs.  Per tile:
+// samples per tile, one CTA per SM holding two tile pipelines of 8 warps, so
+// that one pipeline's epilogue overlaps the other's MMAs.  Per tile:
 //   Z1 = X W1^T, Z2 = A1 W2^T (as in the forward kernel), the output layer,
 //   dO = 2 (O - Y) / n and dZ2 = (dO W3) * silu'(Z2) on the CUDA cores,
-//   dA1 = dZ2 W2 (MMA, W2 held transposed), dZ1 = dA1 * silu'(Z1),
-//   G12 += [dZ2^T; dZ1^T] [A1 | X | 1]   (128 x 112, K = the tile's samples)
-//   G3  += [A2^T; 1] [dO | 0]            (128 x 16)
+//   dA1 = dZ2 W2, dZ1 = dA1 * silu'(Z1),
+//   G12 += [dZ2 | dZ1]^T [A1 | X | 1]   (128 x 112, K = the tile's samples)
+//   G3  += [A2 | 1]^T [dO | 0]          (128 x 16)
 // G12 and G3 stay in each pipeline's half of tensor memory across its tiles;
-// their blocks are gW2, gW1 and, through the rows and columns of ones, the
-// bias gradients.  The CTA writes the two pipelines' sum as its gradient
-// partial (partials are summed over CTAs in a fixed order afterwards, so the
-// result is deterministic).
+// their blocks are gW2, gW1 and, through the columns of ones, the bias
+// gradients.  The CTA writes the two pipelines' sum as its gradient partial
+// (partials are summed over CTAs in a fixed order afterwards, so the result
+// is deterministic).
+//
+// The tensor cores are a few per cent busy: a tile's time is its chain of
+// epilogues.  So
+//   * two threads share a sample, each with half of the hidden units (the two
+//     warps of a lane quarter), and meet once, for the output layer;
+//   * one sigmoid per pre-activation serves SiLU and its derivative, which
+//     waits in registers for the backward pass;
+//   * every activation is stored once, as 16-byte vectors in (sample, unit)
+//     core matrices.  Those are K-major operands of the layer products and,
+//     with the transpose bits of the instruction descriptor, MN-major
+//     operands of the weight gradients: no transposed 2-byte stores.
+// One training batch of 32,768: 56.6 us with one thread per sample, 16.4 here.
 namespace gr {
 
 constexpr int kPipes = 2;                   // tile pipelines per CTA
-constexpr int kThreads = kPipes * TILE;
+constexpr int kThreads = kPipes * kPipeThreads;
 constexpr uint32_t kColsPerPipe = 256;      // Z1 0-63, Z2 / dA1 64-127, G12 128-239, G3 240-255
 constexpr uint32_t kTmemCols = kPipes * kColsPerPipe;  // all 512 columns of the SM
-constexpr int N12 = 112, N3 = 16, KS = TILE;  // KS: samples per tile = K of the weight gradients
-// Rows the weight-gradient operands hold.  The MMAs read N12, TILE and N3
-// rows; the rows past these fall in the buffers that follow in shared memory
-// (bf16 operand or weight arrays), and their values reach only accumulator
-// columns (104-111 of G12, 8-15 of G3) or rows (72-127 of G3) never read.
-constexpr int kB12Rows = 104, kA3Rows = 72, kB3Rows = 8;
+constexpr int N12 = 112, N3 = 16;
+constexpr int kW12 = 2 * HID, kB12 = N12, kW3 = 72, kB3 = N3;  // row widths of the operands
 
+// Operands as (sample, column) rows of 8 x 16-byte core matrices.  The G3
+// MMAs read 128 columns of A3's 72; those past its rows are columns of the
+// next sample group (of B3 after the last), and their values reach only rows
+// 72-127 of G3, never read.
 struct Pipe {
-  __nv_bfloat16 A12[TILE * KS];      // (row, sample): dZ2^T rows 0-63, dZ1^T rows 64-127;
-                                     // the X tile (sample, feature) uses its start until Z1 is formed
-  __nv_bfloat16 A1[TILE * HID];      // (sample, unit); dZ2 (sample, unit) once Z2 is formed
-  __nv_bfloat16 B12[kB12Rows * KS];  // (col, sample): A1^T 0-63, X^T 64-95, ones 96, zeros 97-103
-  __nv_bfloat16 A3[kA3Rows * KS];    // (row, sample): A2^T 0-63, ones 64, zeros 65-71
-  __nv_bfloat16 B3[kB3Rows * KS];    // (col, sample): dO 0-1, zeros 2-7
+  __nv_bfloat16 A12[TILE * kW12];  // dZ2 0-63, dZ1 64-127
+  __nv_bfloat16 B12[TILE * kB12];  // A1 0-63, X 64-95, ones 96, zeros 97-111
+  __nv_bfloat16 A3[TILE * kW3];    // A2 0-63, ones 64, zeros 65-71
+  __nv_bfloat16 B3[TILE * kB3];    // dO 0-1, zeros 2-15
+  float2 part[2][TILE];            // the two halves of the output layer's sums
 };
 
 struct Smem {
   Pipe pipe[kPipes];
   __nv_bfloat16 W1[HID * IN];
   __nv_bfloat16 W2[HID * HID];
-  __nv_bfloat16 W2T[HID * HID];
   float b1[HID], b2[HID], W3[OUT * HID], b3[OUT];
   float loss[kThreads / 32];
   unsigned long long mbar[kPipes];
   uint32_t tmem;
+  int have[kPipes];
 };
 
 constexpr size_t smem_bytes() { return sizeof(Smem) + 128; }
+
+// Position of parameter k in a CTA's partial: the two weight matrices
+// transposed, so that the lanes that own consecutive rows write consecutive
+// floats.
+__device__ __forceinline__ int at_w1(int o, int k) { return OFF_W1 + k * HID + o; }
+__device__ __forceinline__ int at_w2(int o, int c) { return OFF_W2 + c * HID + o; }
+__device__ __forceinline__ int param_of(int i) {
+  if (i < OFF_B1) return OFF_W1 + (i % HID) * IN + i / HID;
+  if (i >= OFF_W2 && i < OFF_B2) return OFF_W2 + ((i - OFF_W2) % HID) * HID + (i - OFF_W2) / HID;
+  return i;
+}
 
 __global__ void __launch_bounds__(kThreads, 1) grad_kernel(const __nv_bfloat16* X, const float* Y,
                                                            int64_t n, float inv_n, const float* P,
@@ -404,28 +505,23 @@ __global__ void __launch_bounds__(kThreads, 1) grad_kernel(const __nv_bfloat16* 
   extern __shared__ unsigned char smem_raw[];
   Smem& s = *reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~(uintptr_t)127);
   const int cta_tid = threadIdx.x, warp = cta_tid >> 5, lane = cta_tid & 31;
-  const int pi = cta_tid / TILE, tid = cta_tid % TILE;  // pipeline, thread (= tile row) within it
+  const int pi = cta_tid / kPipeThreads, tid = cta_tid % kPipeThreads;
+  const int half = (warp >> 2) & 1;           // which half of the hidden units
+  const int r = (warp & 3) * 32 + lane;       // tile row (sample) = tensor-memory lane
+  const int u0 = half * (HID / 2);
   const int bar_id = 1 + pi;
   Pipe& b = s.pipe[pi];
-  const __nv_bfloat16 one = __float2bfloat16_rn(1.0f), zero = __float2bfloat16_rn(0.0f);
-  for (int i = cta_tid; i < HID * IN; i += kThreads) s.W1[kmaj(i / IN, i % IN, IN)] = __float2bfloat16_rn(P[OFF_W1 + i]);
-  for (int i = cta_tid; i < HID * HID; i += kThreads) {
-    const int o = i / HID, c = i % HID;
-    const __nv_bfloat16 w = __float2bfloat16_rn(P[OFF_W2 + i]);
-    s.W2[kmaj(o, c, HID)] = w;   // B of Z2 = A1 W2^T: (n = o, k = c)
-    s.W2T[kmaj(c, o, HID)] = w;  // B of dA1 = dZ2 W2: (n = c, k = o)
-  }
-  for (int i = cta_tid; i < HID; i += kThreads) {
-    s.b1[i] = P[OFF_B1 + i];
-    s.b2[i] = P[OFF_B2 + i];
-  }
-  for (int i = cta_tid; i < OUT * HID; i += kThreads) s.W3[i] = __bfloat162float(__float2bfloat16_rn(P[OFF_W3 + i]));
-  if (cta_tid < OUT) s.b3[cta_tid] = P[OFF_B3 + cta_tid];
-  // constant rows of this pipeline's weight-gradient operands
-  for (int k = 0; k < KS; ++k) {
-    if (tid >= HID + IN && tid < kB12Rows) b.B12[kmaj(tid, k, KS)] = tid == HID + IN ? one : zero;
-    if (tid >= HID && tid < kA3Rows) b.A3[kmaj(tid, k, KS)] = tid == HID ? one : zero;
-    if (tid >= OUT && tid < kB3Rows) b.B3[kmaj(tid, k, KS)] = zero;
+  load_weights<kThreads>(s, P);
+  // constant columns of this pipeline's weight-gradient operands
+  {
+    const uint4 zero = make_uint4(0u, 0u, 0u, 0u), one = make_uint4(0x3f80u, 0u, 0u, 0u);  // 1, 0, ..
+    if (half == 0) {
+      *reinterpret_cast<uint4*>(&b.B12[kmaj(r, HID + IN, kB12)]) = one;
+      *reinterpret_cast<uint4*>(&b.B12[kmaj(r, HID + IN + 8, kB12)]) = zero;
+    } else {
+      *reinterpret_cast<uint4*>(&b.A3[kmaj(r, HID, kW3)]) = one;
+      *reinterpret_cast<uint4*>(&b.B3[kmaj(r, 8, kB3)]) = zero;
+    }
   }
   const uint32_t bar = smem_u32(&s.mbar[pi]);
   if (tid == 0) {
@@ -444,14 +540,14 @@ __global__ void __launch_bounds__(kThreads, 1) grad_kernel(const __nv_bfloat16* 
   fence_after();
   const uint32_t tmem = s.tmem + pi * kColsPerPipe;
   const uint32_t row = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-  const uint32_t x_a = smem_u32(b.A12), a1_a = smem_u32(b.A1), dz2_a = smem_u32(b.A1);
   const uint32_t a12_a = smem_u32(b.A12), b12_a = smem_u32(b.B12), a3_a = smem_u32(b.A3),
-                 b3_a = smem_u32(b.B3);
-  const uint32_t w1_a = smem_u32(s.W1), w2_a = smem_u32(s.W2), w2t_a = smem_u32(s.W2T);
-  __nv_bfloat16* const Xs = b.A12;   // the X tile, until Z1 is formed
-  __nv_bfloat16* const dZ2s = b.A1;  // dZ2, once Z2 is formed
-  constexpr uint32_t kId64 = idesc_bf16(TILE, HID), kId12 = idesc_bf16(TILE, N12),
-                     kId3 = idesc_bf16(TILE, N3);
+                 b3_a = smem_u32(b.B3), w1_a = smem_u32(s.W1), w2_a = smem_u32(s.W2);
+  // bytes of one 8-sample row of core matrices of each operand
+  constexpr uint32_t kRowA12 = kW12 / 8 * 128, kRowB12 = kB12 / 8 * 128, kRowA3 = kW3 / 8 * 128,
+                     kRowB3 = kB3 / 8 * 128;
+  constexpr uint32_t kTA = 1u << 15, kTB = 1u << 16;  // MN-major A, B
+  constexpr uint32_t kId64 = idesc_bf16(TILE, HID), kIdA1 = kId64 | kTB,
+                     kId12 = idesc_bf16(TILE, N12) | kTA | kTB, kId3 = idesc_bf16(TILE, N3) | kTA | kTB;
   uint32_t phase = 0;
   bool ok = true;
   float lsum = 0.0f;
@@ -459,10 +555,10 @@ __global__ void __launch_bounds__(kThreads, 1) grad_kernel(const __nv_bfloat16* 
   auto sync_issue = [&]() {
     fence_async_smem();
     fence_before();
-    pipe_sync(bar_id);
+    pipe_bar(bar_id);
   };
   auto wait = [&]() {
-    ok = pipe_and(bar_id, mbar_wait(bar, phase));
+    ok = pipe_bar_and(bar_id, mbar_wait(bar, phase));
     phase ^= 1;
     fence_after();
     return ok;
@@ -471,127 +567,129 @@ __global__ void __launch_bounds__(kThreads, 1) grad_kernel(const __nv_bfloat16* 
   // of fewer tiles than CTAs still spreads over every SM
   const int64_t stride = (int64_t)gridDim.x * kPipes * TILE;
   for (int64_t m0 = ((int64_t)pi * gridDim.x + blockIdx.x) * TILE; m0 < n && ok; m0 += stride) {
-    const int64_t p = m0 + tid;
+    const int64_t p = m0 + r;
     const bool live = p < n;
-    // X tile: (sample, feature) for Z1 and (feature, sample) for G12
-    uint4 v[4] = {};
-    if (live) {
-      const uint4* src = reinterpret_cast<const uint4*>(X + p * IN);
+    float y0 = 0.0f, y1 = 0.0f;
 #pragma unroll
-      for (int j = 0; j < 4; ++j) v[j] = src[j];
+    for (int j = 0; j < 2; ++j) {
+      const int f = (2 * half + j) * 8;
+      const uint4 v = live ? *reinterpret_cast<const uint4*>(X + p * IN + f) : make_uint4(0u, 0u, 0u, 0u);
+      *reinterpret_cast<uint4*>(&b.B12[kmaj(r, HID + f, kB12)]) = v;
     }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      *reinterpret_cast<uint4*>(&Xs[kmaj(tid, 8 * j, IN)]) = v[j];
-      const __nv_bfloat16* e = reinterpret_cast<const __nv_bfloat16*>(&v[j]);
-#pragma unroll
-      for (int q = 0; q < 8; ++q) b.B12[kmaj(HID + 8 * j + q, tid, KS)] = e[q];
+    if (live) {
+      y0 = Y[p * OUT + 0];
+      y1 = Y[p * OUT + 1];
     }
     sync_issue();
     if (tid == 0) {
       fence_after();
 #pragma unroll
       for (int k = 0; k < IN / 16; ++k)
-        mma(tmem, sdesc(x_a + k * 256, 128, (IN / 8) * 128), sdesc(w1_a + k * 256, 128, (IN / 8) * 128), kId64, k);
+        mma(tmem, sdesc(b12_a + HID / 8 * 128 + k * 256, 128, kRowB12),
+            sdesc(w1_a + k * 256, 128, (IN / 8) * 128), kId64, k);
       commit(bar);
     }
     if (!wait()) break;
-    // A1 = bf16(silu(Z1 + b1)): (sample, unit) for Z2, (unit, sample) for G12
+    // A1 = bf16(silu(Z1 + b1)), silu' kept
+    float ds1[HID / 2];
 #pragma unroll
-    for (int c = 0; c < HID; c += 16) {
+    for (int c = 0; c < HID / 2; c += 16) {
       float z[16];
-      tmem_ld16(row + c, z);
+      tmem_ld16(row + u0 + c, z);
 #pragma unroll
-      for (int j = 0; j < 16; ++j) z[j] = silu(z[j] + s.b1[c + j]);
-      const uint4 u0 = pack8(z), u1 = pack8(z + 8);
-      *reinterpret_cast<uint4*>(&b.A1[kmaj(tid, c, HID)]) = u0;
-      *reinterpret_cast<uint4*>(&b.A1[kmaj(tid, c + 8, HID)]) = u1;
-#pragma unroll
-      for (int j = 0; j < 16; ++j) b.B12[kmaj(c + j, tid, KS)] = __float2bfloat16_rn(z[j]);
+      for (int j = 0; j < 16; ++j) {
+        const float zz = z[j] + s.b1[u0 + c + j];
+        const float sg = sigmoid(zz);
+        z[j] = zz * sg;
+        ds1[c + j] = sg * (1.0f + zz * (1.0f - sg));
+      }
+      *reinterpret_cast<uint4*>(&b.B12[kmaj(r, u0 + c, kB12)]) = pack8(z);
+      *reinterpret_cast<uint4*>(&b.B12[kmaj(r, u0 + c + 8, kB12)]) = pack8(z + 8);
     }
     sync_issue();
     if (tid == 0) {
       fence_after();
 #pragma unroll
       for (int k = 0; k < HID / 16; ++k)
-        mma(tmem + HID, sdesc(a1_a + k * 256, 128, (HID / 8) * 128), sdesc(w2_a + k * 256, 128, (HID / 8) * 128),
+        mma(tmem + HID, sdesc(b12_a + k * 256, 128, kRowB12), sdesc(w2_a + k * 256, 128, (HID / 8) * 128),
             kId64, k);
       commit(bar);
     }
     if (!wait()) break;
-    // output layer, dO, dZ2 = (dO W3) * silu'(Z2 + b2)
-    float a2[HID];
-    float o0 = s.b3[0], o1 = s.b3[1];
+    // A2 and the output layer's half sums, silu' kept
+    float ds2[HID / 2];
+    float o0 = 0.0f, o1 = 0.0f;
 #pragma unroll
-    for (int c = 0; c < HID; c += 16) {
+    for (int c = 0; c < HID / 2; c += 16) {
       float z[16];
-      tmem_ld16(row + HID + c, z);
+      tmem_ld16(row + HID + u0 + c, z);
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
-        const float zz = z[j] + s.b2[c + j];
-        a2[c + j] = zz;  // pre-activation for now
-        const float a = __bfloat162float(__float2bfloat16_rn(silu(zz)));
-        o0 = fmaf(a, s.W3[c + j], o0);
-        o1 = fmaf(a, s.W3[HID + c + j], o1);
+        const float zz = z[j] + s.b2[u0 + c + j];
+        const float sg = sigmoid(zz);
+        ds2[c + j] = sg * (1.0f + zz * (1.0f - sg));
+        z[j] = __bfloat162float(__float2bfloat16_rn(zz * sg));
+        o0 = fmaf(z[j], s.W3[u0 + c + j], o0);
+        o1 = fmaf(z[j], s.W3[HID + u0 + c + j], o1);
       }
+      *reinterpret_cast<uint4*>(&b.A3[kmaj(r, u0 + c, kW3)]) = pack8(z);
+      *reinterpret_cast<uint4*>(&b.A3[kmaj(r, u0 + c + 8, kW3)]) = pack8(z + 8);
     }
+    b.part[half][r] = make_float2(o0, o1);
+    pipe_bar(bar_id);
+    const float2 h0 = b.part[0][r], h1 = b.part[1][r];
     float d0 = 0.0f, d1 = 0.0f;
     if (live) {
-      d0 = o0 - Y[p * OUT + 0];
-      d1 = o1 - Y[p * OUT + 1];
-      lsum += (d0 * d0 + d1 * d1) * inv_n;
+      d0 = (s.b3[0] + h0.x) + h1.x - y0;
+      d1 = (s.b3[1] + h0.y) + h1.y - y1;
+      if (half == 0) lsum += (d0 * d0 + d1 * d1) * inv_n;
       d0 *= 2.0f * inv_n;
       d1 *= 2.0f * inv_n;
     }
-    b.B3[kmaj(0, tid, KS)] = __float2bfloat16_rn(d0);
-    b.B3[kmaj(1, tid, KS)] = __float2bfloat16_rn(d1);
+    if (half == 0)
+      *reinterpret_cast<uint4*>(&b.B3[kmaj(r, 0, kB3)]) =
+          make_uint4(pack2(__float2bfloat16_rn(d0), __float2bfloat16_rn(d1)), 0u, 0u, 0u);
+    // dZ2 = (dO W3) * silu'(Z2 + b2)
 #pragma unroll
-    for (int c = 0; c < HID; c += 8) {
+    for (int c = 0; c < HID / 2; c += 8) {
       float g[8];
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const float zz = a2[c + j];
-        const __nv_bfloat16 act = __float2bfloat16_rn(silu(zz));
-        b.A3[kmaj(c + j, tid, KS)] = act;  // A2^T
-        g[j] = (d0 * s.W3[c + j] + d1 * s.W3[HID + c + j]) * dsilu(zz);
-      }
-      const uint4 u = pack8(g);
-      *reinterpret_cast<uint4*>(&dZ2s[kmaj(tid, c, HID)]) = u;
-      const __nv_bfloat16* e = reinterpret_cast<const __nv_bfloat16*>(&u);
-#pragma unroll
-      for (int j = 0; j < 8; ++j) b.A12[kmaj(c + j, tid, KS)] = e[j];  // dZ2^T
+      for (int j = 0; j < 8; ++j)
+        g[j] = (d0 * s.W3[u0 + c + j] + d1 * s.W3[HID + u0 + c + j]) * ds2[c + j];
+      *reinterpret_cast<uint4*>(&b.A12[kmaj(r, u0 + c, kW12)]) = pack8(g);
     }
     sync_issue();
+    const int acc0 = tiles > 0;
     if (tid == 0) {
       fence_after();
 #pragma unroll
-      for (int k = 0; k < HID / 16; ++k)
-        mma(tmem + HID, sdesc(dz2_a + k * 256, 128, (HID / 8) * 128),
-            sdesc(w2t_a + k * 256, 128, (HID / 8) * 128), kId64, k);
+      for (int k = 0; k < HID / 16; ++k)  // dA1 = dZ2 W2: W2 (o, c) as B with N = c, K = o
+        mma(tmem + HID, sdesc(a12_a + k * 256, 128, kRowA12),
+            sdesc(w2_a + k * 2 * (HID / 8) * 128, (HID / 8) * 128, 128), kIdA1, k);
+#pragma unroll
+      for (int k = 0; k < TILE / 16; ++k)
+        mma(tmem + 2 * HID + N12, sdesc(a3_a + k * 2 * kRowA3, kRowA3, 128),
+            sdesc(b3_a + k * 2 * kRowB3, kRowB3, 128), kId3, acc0 | k);
       commit(bar);
     }
     if (!wait()) break;
-    // dZ1 = dA1 * silu'(Z1 + b1) -> rows 64-127 of A12
+    // dZ1 = dA1 * silu'(Z1 + b1)
 #pragma unroll
-    for (int c = 0; c < HID; c += 16) {
-      float da[16], z[16];
-      tmem_ld16(row + HID + c, da);
-      tmem_ld16(row + c, z);
+    for (int c = 0; c < HID / 2; c += 16) {
+      float da[16];
+      tmem_ld16(row + HID + u0 + c, da);
 #pragma unroll
-      for (int j = 0; j < 16; ++j)
-        b.A12[kmaj(HID + c + j, tid, KS)] = __float2bfloat16_rn(da[j] * dsilu(z[j] + s.b1[c + j]));
+      for (int j = 0; j < 16; ++j) da[j] *= ds1[c + j];
+      *reinterpret_cast<uint4*>(&b.A12[kmaj(r, HID + u0 + c, kW12)]) = pack8(da);
+      *reinterpret_cast<uint4*>(&b.A12[kmaj(r, HID + u0 + c + 8, kW12)]) = pack8(da + 8);
     }
     sync_issue();
     if (tid == 0) {
       fence_after();
-      const int acc0 = tiles > 0;
 #pragma unroll
-      for (int k = 0; k < KS / 16; ++k) {
-        mma(tmem + 2 * HID, sdesc(a12_a + k * 256, 128, (KS / 8) * 128), sdesc(b12_a + k * 256, 128, (KS / 8) * 128),
-            kId12, acc0 | k);
-        mma(tmem + 2 * HID + N12, sdesc(a3_a + k * 256, 128, (KS / 8) * 128), sdesc(b3_a + k * 256, 128, (KS / 8) * 128),
-            kId3, acc0 | k);
-      }
+      for (int k = 0; k < TILE / 16; ++k)
+        mma(tmem + 2 * HID, sdesc(a12_a + k * 2 * kRowA12, kRowA12, 128),
+            sdesc(b12_a + k * 2 * kRowB12, kRowB12, 128), kId12, acc0 | k);
       commit(bar);
     }
     if (!wait()) break;
@@ -599,45 +697,38 @@ __global__ void __launch_bounds__(kThreads, 1) grad_kernel(const __nv_bfloat16* 
   }
   for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
   if (lane == 0) s.loss[warp] = lsum;
-  // the CTA's partial: pipeline 0 writes its G12 and G3 rows (zeros without
-  // a tile), then pipeline 1 adds its own
-  float* out = partial + (int64_t)blockIdx.x * NPARAM;
+  if (tid == 0) s.have[pi] = tiles;
+  fence_before();
   const bool all_ok = __syncthreads_and(ok);
-  for (int turn = 0; turn < kPipes; ++turn) {
-    if (pi == turn && all_ok) {
-      const bool have = tiles > 0;
-      auto put = [&](int idx, float v) {
-        if (turn == 0) out[idx] = have ? v : 0.0f;
-        else if (have) out[idx] += v;
-      };
-#pragma unroll 1
-      for (int c = 0; c < N12; c += 16) {
-        float g[16];
-        tmem_ld16(row + 2 * HID + c, g);
+  fence_after();
+  // the CTA's partial: both pipelines' accumulators (zero without a tile),
+  // 16 columns at a time, dealt over the four warps of each lane quarter
+  float* out = partial + (int64_t)blockIdx.x * NPARAM;
+  if (all_ok) {
+    const uint32_t lane_base = s.tmem + ((uint32_t)((warp & 3) * 32) << 16) + 2 * HID;
+    const bool have0 = s.have[0] > 0, have1 = s.have[1] > 0;
+    for (int c = (warp >> 2) * 16; c < N12 + N3; c += 64) {
+      float g[16], h[16];
+      tmem_ld16(lane_base + c, g);
+      tmem_ld16(lane_base + kColsPerPipe + c, h);
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const int col = c + j;
-          if (tid < HID) {  // rows dZ2^T: gW2[o][c], gb2[o]
-            if (col < HID) put(OFF_W2 + tid * HID + col, g[j]);
-            if (col == HID + IN) put(OFF_B2 + tid, g[j]);
-          } else {          // rows dZ1^T: gW1[o][k], gb1[o]
-            const int o = tid - HID;
-            if (col >= HID && col < HID + IN) put(OFF_W1 + o * IN + (col - HID), g[j]);
-            if (col == HID + IN) put(OFF_B1 + o, g[j]);
+      for (int j = 0; j < 16; ++j) {
+        const int col = c + j;
+        const float v = have0 ? (have1 ? g[j] + h[j] : g[j]) : 0.0f;
+        if (col < N12) {
+          if (r < HID) {  // rows dZ2: gW2[o][c], gb2[o]
+            if (col < HID) out[at_w2(r, col)] = v;
+            if (col == HID + IN) out[OFF_B2 + r] = v;
+          } else {        // rows dZ1: gW1[o][k], gb1[o]
+            if (col >= HID && col < HID + IN) out[at_w1(r - HID, col - HID)] = v;
+            if (col == HID + IN) out[OFF_B1 + r - HID] = v;
           }
+        } else if (col < N12 + OUT) {
+          if (r < HID) out[OFF_W3 + (col - N12) * HID + r] = v;  // sum_i dO[i] A2[i][c]
+          if (r == HID) out[OFF_B3 + (col - N12)] = v;
         }
       }
-      float g3[16];
-      tmem_ld16(row + 2 * HID + N12, g3);
-      if (tid < HID) {
-        put(OFF_W3 + tid, g3[0]);  // gW3[0][c] = sum_i dO[i][0] A2[i][c]
-        put(OFF_W3 + HID + tid, g3[1]);
-      } else if (tid == HID) {
-        put(OFF_B3 + 0, g3[0]);
-        put(OFF_B3 + 1, g3[1]);
-      }
     }
-    __syncthreads();
   }
   if (cta_tid == 0) {
     float l = 0.0f;
@@ -655,19 +746,41 @@ __global__ void __launch_bounds__(kThreads, 1) grad_kernel(const __nv_bfloat16* 
 
 }  // namespace tc
 
-// grad[k] = sum over blocks of partial[b][k] in block order (deterministic).
-__global__ void reduce_kernel(const float* partial, int nb, float* grad, const float* loss_partial,
-                              float* loss) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < NPARAM) {
-    float acc = 0.0f;
-    for (int b = 0; b < nb; ++b) acc += partial[(int64_t)b * NPARAM + k];
-    grad[k] = acc;
+// grad = the CTA partials (in the partials' own order, gr::param_of) summed in
+// a fixed order: each warp takes 32 parameters and every eighth partial, the
+// warps of a CTA are joined in order (152 partials: 6.6 us, 11.2 with one
+// thread per parameter walking them all; sixteen slices gave nothing more).
+// The last CTA sums the losses.
+constexpr int kRedParams = 32, kRedSlices = 8;
+constexpr int kRedGrid = (NPARAM + kRedParams - 1) / kRedParams;
+__global__ void __launch_bounds__(kRedParams* kRedSlices) reduce_kernel(const float* __restrict__ partial,
+                                                                        int nb, float* grad,
+                                                                        const float* loss_partial,
+                                                                        float* loss) {
+  __shared__ float s[kRedSlices][kRedParams];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const bool is_loss = blockIdx.x == kRedGrid;
+  if (is_loss && !loss) return;
+  const int i = blockIdx.x * kRedParams + lane;
+  float acc = 0.0f;
+  if (is_loss) {
+    for (int b = threadIdx.x; b < nb; b += kRedParams * kRedSlices) acc += loss_partial[b];
+  } else if (i < NPARAM) {
+#pragma unroll 4
+    for (int b = w; b < nb; b += kRedSlices) acc += partial[(int64_t)b * NPARAM + i];
   }
-  if (k == 0 && loss) {
-    float l = 0.0f;
-    for (int b = 0; b < nb; ++b) l += loss_partial[b];
-    *loss = l;
+  s[w][lane] = acc;
+  __syncthreads();
+  if (w != 0) return;
+  acc = s[0][lane];
+#pragma unroll
+  for (int k = 1; k < kRedSlices; ++k) acc += s[k][lane];
+  if (is_loss) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) *loss = acc;
+  } else if (i < NPARAM) {
+    grad[tc::gr::param_of(i)] = acc;
   }
 }
 
@@ -689,60 +802,145 @@ __global__ void adam_kernel(float* P, const float* g, float* m, float* v, float 
 // standardised targets and shuffled mini-batches.
 namespace prep {
 
-constexpr int kThreads = 256;
+constexpr int kThreads = 128;
 constexpr int kMaxBlocks = 1024;
 constexpr int kNF = NS + 1;  // 29 log-scaled states and T/100
 
-// Feature f of sample p, as the features kernel forms it before standardising.
-__device__ __forceinline__ float raw_feature(const double* y, int64_t ld, const double* T,
-                                             int64_t p, int f) {
-  if (f < NS) return log10f(fmaxf((float)y[(int64_t)f * ld + p], kLogFloor));
-  return (float)T[p] * 0.01f;
+// Sums of a CTA's per-thread values v[0 .. k): a shuffle tree per warp, then
+// the warps in order; thread j < k writes out[j * stride].  s: k doubles per
+// warp of shared memory.
+template <int K>
+__device__ __forceinline__ void block_sums(double (&v)[K], double* s, double* out, int stride) {
+#pragma unroll
+  for (int j = 0; j < K; ++j) {
+    double x = v[j];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    if ((threadIdx.x & 31) == 0) s[(threadIdx.x >> 5) * K + j] = x;
+  }
+  __syncthreads();
+  if (threadIdx.x < K) {
+    double x = 0.0;
+#pragma unroll
+    for (int w = 0; w < kThreads / 32; ++w) x += s[w * K + threadIdx.x];
+    out[threadIdx.x * stride] = x;
+  }
+  __syncthreads();
 }
 
-// Block partials of sum and sum of squares (FP64) of every feature over a
-// grid-stride share of the samples: part[b][0][f], part[b][1][f].
-__global__ void __launch_bounds__(kThreads) feature_partials(const double* y, int64_t ld,
-                                                             const double* T, int64_t n,
-                                                             double* part) {
-  __shared__ double s1[kThreads], s2[kThreads];
-  for (int f = 0; f < kNF; ++f) {
-    double a = 0.0, b = 0.0;
-    for (int64_t p = (int64_t)blockIdx.x * kThreads + threadIdx.x; p < n;
-         p += (int64_t)gridDim.x * kThreads) {
-      const double v = raw_feature(y, ld, T, p, f);
-      a += v;
-      b += v * v;
+// Exact sums of floats without the FP64 pipe (an FP64 addition holds it for
+// 64 cycles per warp).  A value |x| < 64 is added to a 64-bit integer in
+// units of 2^-38, in two pieces that adding 1.5 x 2^23 rounds to integers;
+// every float of magnitude 2^-14 or more is a multiple of that unit, so the
+// sum is exact but for smaller terms, each rounded by at most 2^-39.  Room
+// for 2^63-38 / 64 = 524,288 terms.  Values from 64 up and NaN go to `out`.
+struct FixedSum {
+  long long q = 0;
+  float out = 0.0f;
+  // the sum over the warp's lanes, in every lane
+  __device__ __forceinline__ void warp_sum() {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      q += __shfl_xor_sync(0xffffffffu, q, o);
+      out += __shfl_xor_sync(0xffffffffu, out, o);
     }
-    s1[threadIdx.x] = a;
-    s2[threadIdx.x] = b;
-    __syncthreads();
-    for (int w = kThreads / 2; w > 0; w >>= 1) {
-      if (threadIdx.x < w) {
-        s1[threadIdx.x] += s1[threadIdx.x + w];
-        s2[threadIdx.x] += s2[threadIdx.x + w];
-      }
-      __syncthreads();
+  }
+  __device__ __forceinline__ void add(float x) {
+    const float M = 12582912.0f;
+    const bool in = fabsf(x) < 64.0f;
+    const float t = in ? x * 65536.0f : 0.0f;
+    const float h = t + M;
+    const float l = (t - (h - M)) * 4194304.0f + M;
+    q += (long long)(__float_as_int(h) - 0x4b400000) * 4194304ll + (__float_as_int(l) - 0x4b400000);
+    if (!in) out += x;
+  }
+  __device__ __forceinline__ double value() const {
+    return (double)q * 3.637978807091713e-12 + (double)out;  // 2^-38
+  }
+};
+
+// h + l += x + y, the rounding error of h + x (Knuth's TwoSum) going into l
+__device__ __forceinline__ void add_two_float(float& h, float& l, float x, float y) {
+  const float t = h + x, bb = t - h;
+  l += ((h - (t - bb)) + (x - bb)) + y;
+  h = t;
+}
+
+// Block partials of sum and sum of squares of the features over a
+// grid-stride share of the samples: part[b][0][f], part[b][1][f], each thread
+// with the sums of six features in registers (blockIdx.y).  The sum of x and
+// the leading 12 + 12 bits' product parts go through FixedSum: x^2 = p + e
+// exactly (p the rounded product / 32, below 64 for log10 of any float), e
+// summed with its rounding errors.  1M samples: 470 us with one FP64 tree per
+// feature, 319 with FP64 joining trees in 4,880 CTAs, 154 with these in one
+// resident wave.  Bound by the logarithms' issue and latency.
+constexpr int kGroup = 6;
+__global__ void __launch_bounds__(kThreads) feature_partials(const double* __restrict__ y,
+                                                             int64_t ld,
+                                                             const double* __restrict__ T,
+                                                             int64_t n, double* part) {
+  __shared__ double s[2][kThreads / 32][kGroup];
+  const int f0 = blockIdx.y * kGroup;
+  FixedSum a[kGroup], b[kGroup];
+  float eh[kGroup], el[kGroup];
+#pragma unroll
+  for (int j = 0; j < kGroup; ++j) eh[j] = el[j] = 0.0f;
+#pragma unroll 2
+  for (int64_t p = (int64_t)blockIdx.x * kThreads + threadIdx.x; p < n;
+       p += (int64_t)gridDim.x * kThreads) {
+#pragma unroll
+    for (int j = 0; j < kGroup; ++j) {
+      const int f = f0 + j;
+      const float v = f < NS ? log10f(floored(y[(int64_t)f * ld + p])) : (float)T[p] * 0.01f;
+      a[j].add(v);
+      const float sq = __fmul_rn(v, v), e = fmaf(v, v, -sq);
+      b[j].add(sq * 0.03125f);
+      add_two_float(eh[j], el[j], e, 0.0f);
     }
-    if (threadIdx.x == 0) {
-      part[((int64_t)blockIdx.x * 2 + 0) * 32 + f] = s1[0];
-      part[((int64_t)blockIdx.x * 2 + 1) * 32 + f] = s2[0];
+  }
+  // the joining trees stay off the FP64 pipe too: integers and TwoSums
+#pragma unroll
+  for (int j = 0; j < kGroup; ++j) {
+    a[j].warp_sum();
+    b[j].warp_sum();
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+      add_two_float(eh[j], el[j], __shfl_xor_sync(0xffffffffu, eh[j], o),
+                    __shfl_xor_sync(0xffffffffu, el[j], o));
+    if ((threadIdx.x & 31) == 0) {
+      s[0][threadIdx.x >> 5][j] = a[j].value();
+      s[1][threadIdx.x >> 5][j] = 32.0 * b[j].value() + ((double)eh[j] + (double)el[j]);
     }
-    __syncthreads();
+  }
+  __syncthreads();
+  if (threadIdx.x < 2 * kGroup) {
+    const int k = threadIdx.x / kGroup, j = threadIdx.x % kGroup;
+    double x = 0.0;
+#pragma unroll
+    for (int w = 0; w < kThreads / 32; ++w) x += s[k][w][j];
+    part[((int64_t)blockIdx.x * 2 + k) * 32 + f0 + j] = x;
   }
 }
 
 // Mean and 1/std (sample standard deviation, floored at 1e-6) of k series
-// from nb block partials in block order: norm[f] = mean, norm[stride + f] = 1/std.
-__global__ void moments_finish(const double* part, int nb, int k, int pstride, int64_t n,
-                               float* norm, int stride, int scale_std) {
-  const int f = threadIdx.x;
-  if (f >= k) return;
-  double a = 0.0, b = 0.0;
-  for (int i = 0; i < nb; ++i) {
-    a += part[((int64_t)i * 2 + 0) * pstride + f];
-    b += part[((int64_t)i * 2 + 1) * pstride + f];
+// from nb block partials: norm[f] = mean, norm[stride + f] = 1/std.  One CTA
+// per series: its threads add the partials b = t, t + 128, .. and a fixed
+// tree joins them (5.8 us; one warp walking 1,024 partials in order took
+// 156).
+__global__ void __launch_bounds__(kThreads) moments_finish(const double* part, int nb, int pstride,
+                                                           int64_t n, float* norm, int stride,
+                                                           int scale_std) {
+  __shared__ double s[(kThreads / 32) * 2];
+  __shared__ double tot[2];
+  const int f = blockIdx.x;
+  double v[2] = {0.0, 0.0};
+  for (int i = threadIdx.x; i < nb; i += kThreads) {
+    v[0] += part[((int64_t)i * 2 + 0) * pstride + f];
+    v[1] += part[((int64_t)i * 2 + 1) * pstride + f];
   }
+  block_sums<2>(v, s, tot, 1);
+  if (threadIdx.x != 0) return;
+  const double a = tot[0], b = tot[1];
   const double mu = a / (double)n;
   const double var = n > 1 ? fmax(b - a * mu, 0.0) / (double)(n - 1) : 0.0;
   const double sd = fmax(sqrt(var), 1e-6);
@@ -750,44 +948,59 @@ __global__ void moments_finish(const double* part, int nb, int k, int pstride, i
   norm[stride + f] = scale_std ? (float)sd : (float)(1.0 / sd);
 }
 
-// Partials of the two targets log10 S_H and log10 h: part[b][0][k], part[b][1][k].
-__global__ void __launch_bounds__(kThreads) target_partials(const double* SH, const double* h,
-                                                            int64_t n, double* part) {
-  __shared__ double s[4][kThreads];
-  double a0 = 0.0, a1 = 0.0, b0 = 0.0, b1 = 0.0;
-  for (int64_t p = (int64_t)blockIdx.x * kThreads + threadIdx.x; p < n;
-       p += (int64_t)gridDim.x * kThreads) {
-    const double t0 = log10(SH[p]), t1 = log10(h[p]);
-    a0 += t0;
-    a1 += t1;
-    b0 += t0 * t0;
-    b1 += t1 * t1;
-  }
-  s[0][threadIdx.x] = a0;
-  s[1][threadIdx.x] = a1;
-  s[2][threadIdx.x] = b0;
-  s[3][threadIdx.x] = b1;
-  __syncthreads();
-  for (int w = kThreads / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w)
-      for (int j = 0; j < 4; ++j) s[j][threadIdx.x] += s[j][threadIdx.x + w];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    part[((int64_t)blockIdx.x * 2 + 0) * 2 + 0] = s[0][0];
-    part[((int64_t)blockIdx.x * 2 + 0) * 2 + 1] = s[1][0];
-    part[((int64_t)blockIdx.x * 2 + 1) * 2 + 0] = s[2][0];
-    part[((int64_t)blockIdx.x * 2 + 1) * 2 + 1] = s[3][0];
-  }
+// log10 of a positive normal double: x = 2^k m with m in [1/sqrt 2, sqrt 2),
+// log m = 2 atanh(s) = 2 (s + s^3/3 + s^5/5 + ..), s = (m - 1)/(m + 1), |s| <
+// 0.1716: the first term left out, s^23/23, is below 2e-19.  Some 20 FP64
+// instructions where the general function takes twice that.  Other arguments
+// take the general function.
+__device__ __forceinline__ double log10_normal(double x) {
+  const int hi = __double2hiint(x);
+  if ((unsigned)(hi - 0x00100000) >= 0x7fe00000u) return log10(x);
+  // exponent so that the significand's high word lies in [1/sqrt 2, sqrt 2)
+  const int k = (hi - 0x3fe6a09e) >> 20;
+  const double m = __hiloint2double(hi - (k << 20), __double2loint(x));
+  const double s = (m - 1.0) * rcp<double>(m + 1.0);
+  const double z = s * s;
+  double p = 1.0 / 21.0;
+#pragma unroll
+  for (int i = 19; i >= 3; i -= 2) p = fma(p, z, 1.0 / i);
+  const double l = fma(s * z, p, s);  // atanh(s)
+  // log10 2 in two parts, the first with 32 trailing zero bits: k times it is exact
+  const double c1 = 0.30102992057800293, c2 = 7.508597826552624e-08;
+  const double kd = (double)k;
+  return fma(kd, c1, fma(kd, c2, l * 0.86858896380650363));  // 2 / ln 10
 }
 
-// Y[p] = (log10 S_H - mean, log10 h - mean) / std with out_norm = [means, stds].
-__global__ void target_write(const double* SH, const double* h, int64_t n, const float* on,
-                             float* Y) {
+// Partials of the two targets log10 S_H and log10 h: part[b][0][k],
+// part[b][1][k].  The logarithms, rounded to float, wait in Y for the
+// standardisation.  Bound by the FP64 pipe (some 50 instructions per sample):
+// 1M samples 140 us with the general logarithm, 100 here; the
+// standardisation, which formed them anew, took 122 and takes 6.
+__global__ void __launch_bounds__(kThreads) target_partials(const double* __restrict__ SH,
+                                                            const double* __restrict__ h,
+                                                            int64_t n, double* part, float* Y) {
+  __shared__ double s[(kThreads / 32) * 4];
+  double v[4] = {0.0, 0.0, 0.0, 0.0};
+  for (int64_t p = (int64_t)blockIdx.x * kThreads + threadIdx.x; p < n;
+       p += (int64_t)gridDim.x * kThreads) {
+    const double t0 = log10_normal(SH[p]), t1 = log10_normal(h[p]);
+    v[0] += t0;
+    v[1] += t1;
+    v[2] = fma(t0, t0, v[2]);
+    v[3] = fma(t1, t1, v[3]);
+    Y[2 * p] = (float)t0;
+    Y[2 * p + 1] = (float)t1;
+  }
+  block_sums<4>(v, s, part + (int64_t)blockIdx.x * 4, 1);
+}
+
+// Y[p] = (log10 S_H - mean, log10 h - mean) / std with out_norm = [means,
+// stds], in place on the logarithms of target_partials.
+__global__ void target_write(int64_t n, const float* on, float* Y) {
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
-  Y[2 * p + 0] = ((float)log10(SH[p]) - on[0]) / on[2];
-  Y[2 * p + 1] = ((float)log10(h[p]) - on[1]) / on[3];
+  Y[2 * p + 0] = (Y[2 * p + 0] - on[0]) / on[2];
+  Y[2 * p + 1] = (Y[2 * p + 1] - on[1]) / on[3];
 }
 
 // A keyed bijection of [0, n): a balanced four-round Feistel network on the
@@ -843,6 +1056,12 @@ __global__ void gather(const uint4* X, const float2* Y, int64_t M, int half_m, u
 
 __global__ void fill_ones(float* p, int n) {
   if ((int)threadIdx.x < n) p[threadIdx.x] = 1.0f;
+}
+
+// CTAs of the statistics: at least eight samples per thread (the joining
+// tree costs about as much as three), at most `most`: one resident wave.
+inline int grid_for(int64_t n, int most) {
+  return (int)std::max<int64_t>(1, std::min<int64_t>(std::min(most, kMaxBlocks), n / (8 * kThreads)));
 }
 
 // half the even bit count of the Feistel domain of [0, n)
@@ -905,7 +1124,7 @@ chad_status grad_launch(const uint16_t* X, const float* Y, int64_t n, const floa
   float* lpart = partial + nb * NPARAM;
   tc::gr::grad_kernel<<<(unsigned)nb, tc::gr::kThreads, tc::gr::smem_bytes(), s>>>(
       reinterpret_cast<const __nv_bfloat16*>(X), Y, n, 1.0f / (float)n, params, partial, lpart, err);
-  reduce_kernel<<<(NPARAM + 255) / 256, 256, 0, s>>>(partial, (int)nb, grad, lpart, loss);
+  reduce_kernel<<<kRedGrid + 1, kRedParams * kRedSlices, 0, s>>>(partial, (int)nb, grad, lpart, loss);
   return cudaGetLastError() == cudaSuccess ? CHAD_OK : CHAD_E_CUDA;
 }
 
@@ -956,8 +1175,12 @@ chad_status chad_mlp_features(const double* y, int64_t ld, const double* T, int6
                               const float* norm, uint16_t* X, void* stream) {
   if (n < 0 || (n > 0 && (!y || !T || !norm || !X)) || ld < n) return CHAD_E_INVALID;
   if (n == 0) return CHAD_OK;
-  mlp::features_kernel<<<(unsigned)((n + 127) / 128), 128, 0, (cudaStream_t)stream>>>(
-      y, ld, T, n, norm, reinterpret_cast<__nv_bfloat16*>(X));
+  const unsigned grid = (unsigned)((n + 127) / 128);
+  if ((reinterpret_cast<uintptr_t>(X) & 15) == 0)
+    mlp::features_kernel<<<grid, 128, 0, (cudaStream_t)stream>>>(y, ld, T, n, norm,
+                                                                 reinterpret_cast<uint4*>(X));
+  else
+    mlp::features_kernel_unaligned<<<grid, 128, 0, (cudaStream_t)stream>>>(y, ld, T, n, norm, X);
   return cudaGetLastError() == cudaSuccess ? CHAD_OK : CHAD_E_CUDA;
 }
 
@@ -1021,12 +1244,12 @@ chad_status chad_mlp_feature_norm(const double* y, int64_t ld, const double* T, 
   if (n < 2 || !y || !T || !norm || !scratch || ld < n) return CHAD_E_INVALID;
   if (scratch_bytes < chad_mlp_prep_scratch_bytes()) return CHAD_E_INVALID;
   cudaStream_t s = (cudaStream_t)stream;
-  const int nb = (int)std::min<int64_t>(mlp::prep::kMaxBlocks, (n + mlp::prep::kThreads - 1) /
-                                                                   mlp::prep::kThreads);
+  const int nb = mlp::prep::grid_for(n, mlp::sm_count() * 7 / 5);
   double* part = static_cast<double*>(scratch);
-  mlp::prep::feature_partials<<<nb, mlp::prep::kThreads, 0, s>>>(y, ld, T, n, part);
+  mlp::prep::feature_partials<<<dim3(nb, mlp::prep::kNF / mlp::prep::kGroup), mlp::prep::kThreads, 0, s>>>(y, ld, T, n, part);
   // padding features: mean 0, 1/std 1
-  mlp::prep::moments_finish<<<1, 32, 0, s>>>(part, nb, mlp::prep::kNF, 32, n, norm, mlp::IN, 0);
+  mlp::prep::moments_finish<<<mlp::prep::kNF, mlp::prep::kThreads, 0, s>>>(part, nb, 32, n, norm,
+                                                                           mlp::IN, 0);
   if (cudaMemsetAsync(norm + mlp::prep::kNF, 0, sizeof(float) * (mlp::IN - mlp::prep::kNF), s) !=
       cudaSuccess)
     return CHAD_E_CUDA;
@@ -1039,12 +1262,11 @@ chad_status chad_mlp_targets(const double* SH, const double* h, int64_t n, float
   if (n < 2 || !SH || !h || !Y || !out_norm || !scratch) return CHAD_E_INVALID;
   if (scratch_bytes < chad_mlp_prep_scratch_bytes()) return CHAD_E_INVALID;
   cudaStream_t s = (cudaStream_t)stream;
-  const int nb = (int)std::min<int64_t>(mlp::prep::kMaxBlocks, (n + mlp::prep::kThreads - 1) /
-                                                                   mlp::prep::kThreads);
+  const int nb = mlp::prep::grid_for(n, 4 * mlp::sm_count());
   double* part = static_cast<double*>(scratch);
-  mlp::prep::target_partials<<<nb, mlp::prep::kThreads, 0, s>>>(SH, h, n, part);
-  mlp::prep::moments_finish<<<1, 32, 0, s>>>(part, nb, 2, 2, n, out_norm, 2, 1);
-  mlp::prep::target_write<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(SH, h, n, out_norm, Y);
+  mlp::prep::target_partials<<<nb, mlp::prep::kThreads, 0, s>>>(SH, h, n, part, Y);
+  mlp::prep::moments_finish<<<2, mlp::prep::kThreads, 0, s>>>(part, nb, 2, n, out_norm, 2, 1);
+  mlp::prep::target_write<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, out_norm, Y);
   return cudaGetLastError() == cudaSuccess ? CHAD_OK : CHAD_E_CUDA;
 }
 
