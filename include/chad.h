@@ -156,7 +156,8 @@ const char* chad_param_name(int i);
 
 /* Create a context on the current CUDA device.  Validates cfg, derives the
    per-digester model constants (Sec. 2.2; temperature-independent part), and
-   allocates the particle buffers (about 280 bytes per particle in FP64 SoA).
+   allocates the particle buffers (about 280 bytes per particle in FP64 SoA,
+   and up to 96 bytes per resident GPU thread of scratch).
    On error *out is NULL and nothing is leaked. */
 chad_status chad_create(const chad_config* cfg, chad_ctx** out);
 

@@ -88,6 +88,7 @@ struct chad_ctx {
   double* d_atol = nullptr;
   DevCounters* d_cnt = nullptr;
   unsigned long long* d_queue = nullptr;
+  Migrant* d_mig = nullptr;    // particles on their way between threads (integrator tail)
   int* d_order = nullptr;      // [N] queue position -> particle, heaviest first
   int* d_order_cnt = nullptr;  // [2 * kOrderBuckets] bucket counts and cursors
   unsigned long long* d_misc = nullptr;  // [2]: load check flag, failed-particle count
@@ -176,7 +177,7 @@ static DiffArgs diff_args(const chad_ctx* c) {
 
 static void free_all(chad_ctx* c) {
   void* ptrs[] = {c->d_dc, c->d_dcf, c->d_fl, c->d_dig, c->d_off, c->d_y, c->d_pos, c->d_T, c->d_pc, c->d_D,
-                  c->d_SH, c->d_h, c->d_status, c->d_atol, c->d_cnt, c->d_queue, c->d_order, c->d_order_cnt, c->d_misc, c->d_interval, c->d_chunk_dig,
+                  c->d_SH, c->d_h, c->d_status, c->d_atol, c->d_cnt, c->d_queue, c->d_mig, c->d_order, c->d_order_cnt, c->d_misc, c->d_interval, c->d_chunk_dig,
                   c->d_chunk_beg, c->d_chunk_end, c->d_dig_chunk0, c->d_partial, c->d_mean};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -270,12 +271,10 @@ chad_status chad_create(const chad_config* cfg, chad_ctx** out) {
   c->diff_D.assign(c->n_dig, 0.0);
   c->diff_h.assign(c->n_dig, 0.0);
   c->loaded.assign(c->n_dig, 0);
-  {
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    for (int f = 0; f < 5; ++f) c->variant[f] = default_variant(f, c->N, sms);
-  }
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  for (int f = 0; f < 5; ++f) c->variant[f] = default_variant(f, c->N, sms);
   for (int d = 0; d < c->n_dig; ++d) {
     const char* why = "";
     const double Du = cfg->D_uniform ? cfg->D_uniform[d] : 0.0;
@@ -320,6 +319,7 @@ chad_status chad_create(const chad_config* cfg, chad_ctx** out) {
   A(dalloc(&c->d_atol, NS));
   A(dalloc(&c->d_cnt, 1));
   A(dalloc(&c->d_queue, 1));
+  A(dalloc(&c->d_mig, (size_t)migrant_capacity(c->N, sms)));
   A(dalloc(&c->d_order, c->N));
   A(dalloc(&c->d_order_cnt, 2 * kOrderBuckets));
   A(dalloc(&c->d_misc, 2));
@@ -862,6 +862,7 @@ static cudaError_t enqueue_interval(chad_ctx* c, double dt_days, int variant, cu
   a.SH_learned = learned_now ? c->d_SH_learned : nullptr;
   a.h_learned = learned_now ? c->d_h_learned : nullptr;
   a.n_dig = c->n_dig;
+  a.mig = c->d_mig;
   cudaError_t e;
   if (learned_now) {
     const float* P = c->d_mlp;

@@ -138,7 +138,7 @@ __device__ __forceinline__ void wsolve(W w, const float* qv,
 template <int BS, int MINB, bool WS, bool IDX>
 __global__ void __launch_bounds__(BS, MINB) integrate_mx_kernel(StepArgs a) {
   __shared__ unsigned long long s_acc, s_rej, s_newton, s_fb, s_piv, s_redo, s_h2;
-  __shared__ int s_min, s_max;
+  __shared__ int s_min, s_max, warp_count[BS / 32];
   if (threadIdx.x == 0) {
     s_acc = s_rej = s_newton = s_fb = s_piv = s_redo = s_h2 = 0ull;
     s_min = INT_MAX;
@@ -187,7 +187,54 @@ __global__ void __launch_bounds__(BS, MINB) integrate_mx_kernel(StepArgs a) {
   Cnt cnt{0, 0, 0, 0, 0, 0, 0};
 
   bool exhausted = false;
+  int working = BS / 32, live = BS;  // warps with particles; particles at the last attempt
   while (true) {
+    if (BS > 32 && BS < 256 && working > 1 && live <= working * 16) {  // see rank_in_block
+      int total;
+      const int place = rank_in_block<BS>(p >= 0, warp_count, total);
+      Migrant* mig = a.mig + (int64_t)blockIdx.x * BS;
+      if (p >= 0) {
+        Migrant& m = mig[place];
+        m.p = p;
+        m.SH = SHg;
+        m.SH2 = SH2g;
+        m.h = h;
+        m.t = t;
+        m.status = status;
+        m.attempts = attempts;
+        m.nacc = nacc;
+        m.rejected_prev = rejected_prev;
+        pack_counts(cnt, m.counts);
+#pragma unroll
+        for (int i = 0; i < NS; ++i) a.y[i * a.ld + p] = y[i];
+      }
+      __syncthreads();
+      p = -1;
+      if ((int)threadIdx.x < total) {
+        const Migrant& m = mig[threadIdx.x];
+        p = m.p;
+        SHg = m.SH;
+        SH2g = (float)m.SH2;
+        h = m.h;
+        t = m.t;
+        status = m.status;
+        attempts = m.attempts;
+        nacc = m.nacc;
+        rejected_prev = m.rejected_prev != 0;
+        cnt = unpack_counts(m.counts);
+        dg = a.dig[p];
+        c = &a.dc[dg];
+        cf = &a.dcf[dg];
+        pc_load(a.pc, a.ld, p, q);
+        narrow_pc(q, qf);
+        Df = f32(a.D[p]);
+#pragma unroll
+        for (int i = 0; i < NS; ++i) y[i] = a.y[i * a.ld + p];
+        ys_stale = true;  // the float copies are rounded from y again
+      }
+      exhausted = true;
+      working = (total + 31) / 32;
+    }
     bool fresh = false;
     if (p < 0 && !exhausted) {
       p = queue_pop(a.queue);
@@ -245,7 +292,8 @@ __global__ void __launch_bounds__(BS, MINB) integrate_mx_kernel(StepArgs a) {
     // eight warps of an SM in one block: 64 digesters, 400,000 particles,
     // 163 -> 83 ms; 1M particles with slugs 32.9 -> 27.1 ms.  The loop ends
     // when no thread of the block has a particle.
-    if (!__syncthreads_or(p >= 0 || arrived == 0xffffffffu)) break;
+    live = __syncthreads_count(p >= 0 || arrived == 0xffffffffu);
+    if (live == 0) break;
     const bool act = p >= 0;
     // ------------------------------------------------ one step attempt
     bool done = false;

@@ -18,6 +18,15 @@ struct DevCounters {
   unsigned long long h2_iters;  // Eq. 8 Newton iterations (S_h2 algebraic)
 };
 
+// A particle between two attempts, as it moves to another thread of its block
+// (see compact() in integrate_impl.cuh); its states travel through y.
+struct Migrant {
+  long long p;
+  double SH, SH2, h, t;
+  int status, attempts, nacc, rejected_prev;
+  int counts[8];
+};
+
 struct StepArgs {
   int64_t n;            // particles
   int64_t ld;           // leading dimension of the SoA arrays
@@ -43,6 +52,7 @@ struct StepArgs {
   const double* SH_learned;   // learned guesses for particles without history (or null)
   const double* h_learned;
   int n_dig;                  // digesters of the context
+  Migrant* mig;               // [migrant_capacity(n, SMs)] scratch
 };
 
 struct AdvectArgs {
@@ -96,15 +106,19 @@ constexpr KernelVariant kernel_variant(int form, int v) {
 // The variant of a context that asked for none.  Few particles: small blocks
 // spread them over the SMs, so that a warp has its sub-partition's FP64 pipe
 // (one warp instruction per 64 cycles) to itself: 1,000 particles FP64 with
-// S_h2 algebraic 3.23 ms with 128-thread blocks, 2.93 with 32; 20,000
-// particles FP64 11.8 ms against 10.7 with 64.  From about one 160-particle
-// share per SM on, large blocks, whose warps share the fetched code: 45,000
-// particles FP64 15.2 ms with 128 threads, 17.1 with 64.  There form 4 takes
+// S_h2 algebraic 2.92 ms with 128-thread blocks, 2.70 with 64, 2.68 with 32;
+// 12,000 particles FP64 9.72 ms, 9.37, 9.58.  From 128 particles per SM on,
+// large blocks, whose warps share the fetched code: 30,000 particles FP64
+// 11.4 ms with 128 threads, 13.0 with 64.  There form 4 takes
 // one block of eight warps per SM with W_d in shared memory: 64 digesters
 // with 400,000 particles 115.9 ms (128 threads, W_d in registers) against
 // 83.1, 1M particles with slugs 34.0 against 27.1.
 constexpr int default_variant(int form, int64_t n, int sms) {
-  return n <= (int64_t)64 * sms ? 5 : n <= (int64_t)160 * sms ? 3 : form == 4 ? 6 : 0;
+  return n <= (int64_t)64 * sms ? 5 : n <= (int64_t)128 * sms ? 3 : form == 4 ? 6 : 0;
+}
+// Entries of StepArgs::mig: one per resident thread of the persistent grid.
+constexpr int64_t migrant_capacity(int64_t n, int sms) {
+  return n + 256 < (int64_t)sms * 2048 ? n + 256 : (int64_t)sms * 2048;
 }
 cudaError_t launch_integrate(const StepArgs& a, int precision, int variant, cudaStream_t s);
 cudaError_t launch_advect(const AdvectArgs& a, cudaStream_t s);

@@ -868,10 +868,9 @@ __device__ __forceinline__ void add_two_float(float& h, float& l, float x, float
 
 // Block partials of sum and sum of squares of the features over a
 // grid-stride share of the samples: part[b][0][f], part[b][1][f], each thread
-// with the sums of six features in registers (blockIdx.y).  The sum of x and
-// the leading 12 + 12 bits' product parts go through FixedSum: x^2 = p + e
-// exactly (p the rounded product / 32, below 64 for log10 of any float), e
-// summed with its rounding errors.  1M samples: 470 us with one FP64 tree per
+// with the sums of six features in registers (blockIdx.y).  x and p go through
+// FixedSum, where x^2 = p + e exactly with p the rounded square (p / 32 is
+// below 64 for log10 of any float); e is summed with its rounding errors.  1M samples: 470 us with one FP64 tree per
 // feature, 319 with FP64 joining trees in 4,880 CTAs, 154 with these in one
 // resident wave.  Bound by the logarithms' issue and latency.
 constexpr int kGroup = 6;
