@@ -715,6 +715,16 @@ __global__ void __launch_bounds__(BS, MINB) integrate_kernel(StepArgs a) {
               F1[i] = tmp[i];
               tmp[i] = tmp[i] - k1[i];
             }
+          } else if (fixed) {
+            // k3 serves the error estimate alone: of a fixed step only
+            // whether it is finite is asked, here of the rates and the new
+            // solution that it would be formed from (ten fixed substeps of
+            // 111,000 particles: 7.89 -> 6.97 ms)
+            bool fin = true;
+#pragma unroll
+            for (int i = 0; i < NS; ++i) fin = fin && mag64(tmp[i]) < kInfBits && mag64(y1[i]) < kInfBits;
+            norm = fin ? NR(0) : NR(INFINITY);
+            continue;
           } else {
 #pragma unroll
             for (int i = 0; i < NS; ++i)
@@ -742,7 +752,9 @@ __global__ void __launch_bounds__(BS, MINB) integrate_kernel(StepArgs a) {
       }
     }
     if (!act) continue;
-    if (piv_ok || fixed) {
+    if (!MIXED && fixed) {
+      // no error norm (its finiteness: in the last stage)
+    } else if (piv_ok || fixed) {
       // scaled error norm max_i |h/6 (k1 - 2 k2 + k3)_i| / (atol_i + rtol
       // max(|y_i|, |y1_i|)).  FP64 forms: all of it in FP64, as the oracle.
       // Mixed forms: the combination, which cancels, in FP64, everything

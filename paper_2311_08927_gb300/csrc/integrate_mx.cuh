@@ -441,6 +441,10 @@ __global__ void __launch_bounds__(BS, MINB) integrate_mx_kernel(StepArgs a) {
           AcidBase ab;
           Factors<float> k;
           roots(dcn(), dcfn(), q, qf, y1, y1s, Df, SHg, SH2g, a.max_newton, cnt, ab, k);
+          // k3 serves the error estimate alone, and a fixed step has none
+          // (a state that is not finite is flagged when it is stored): ten
+          // substeps of 111,000 particles 4.32 -> 2.76 ms with it
+          if (st == 2 && fixed) continue;
           float Fs[NS];
           rates_f32(dcfn(), qf, y1s, Df, ab, k, Fs);
           if (st == 1) {
