@@ -103,6 +103,13 @@ __device__ __forceinline__ int rank_in_block(bool act, int* warp_count, int& tot
   }
   return rank;
 }
+// The thread that takes place 0: the second half of the grid fills its blocks'
+// last warps instead of the first, so that the blocks that share an SM leave
+// their particles on different sub-partitions.
+template <int BS>
+__device__ __forceinline__ int first_place(int total) {
+  return 2 * blockIdx.x >= gridDim.x ? BS - (total + 31) / 32 * 32 : 0;
+}
 __device__ __forceinline__ void pack_counts(const Cnt& c, int* v) {
   v[0] = c.acc; v[1] = c.rej; v[2] = c.newton; v[3] = c.fallback;
   v[4] = c.failed; v[5] = c.pivot; v[6] = c.redo; v[7] = c.h2;
@@ -456,8 +463,9 @@ __global__ void __launch_bounds__(BS, MINB) integrate_kernel(StepArgs a) {
       }
       __syncthreads();
       p = -1;
-      if ((int)threadIdx.x < total) {
-        const Migrant& m = mig[threadIdx.x];
+      const int at = (int)threadIdx.x - first_place<BS>(total);
+      if (at >= 0 && at < total) {
+        const Migrant& m = mig[at];
         p = m.p;
         SHg = m.SH;
         SH2g = m.SH2;

@@ -210,8 +210,9 @@ __global__ void __launch_bounds__(BS, MINB) integrate_mx_kernel(StepArgs a) {
       }
       __syncthreads();
       p = -1;
-      if ((int)threadIdx.x < total) {
-        const Migrant& m = mig[threadIdx.x];
+      const int at = (int)threadIdx.x - first_place<BS>(total);
+      if (at >= 0 && at < total) {
+        const Migrant& m = mig[at];
         p = m.p;
         SHg = m.SH;
         SH2g = (float)m.SH2;
