@@ -392,8 +392,8 @@ static cudaMemcpyKind kind_in(int mem) { return mem == CHAD_MEM_DEVICE ? cudaMem
 // context array (pitch ld), in either direction.  Device arrays: one 2-D copy
 // for all rows, where a copy per row cost some 2 us of the host's time each
 // (64 digesters with 400,000 particles: some 4,000 of them per load, step and
-// read, 84 -> 67 ms).  Host arrays, and
-// pitches a 2-D copy does not take, row by row.
+// read, 84 -> 67 ms).  Host arrays, and pitches that a 2-D copy does not take,
+// row by row.
 static cudaError_t copy_rows(double* dst, size_t dpitch, const double* src, size_t spitch, int64_t n,
                              int rows, cudaMemcpyKind k, cudaStream_t s) {
   constexpr size_t kMaxPitch = (size_t(1) << 31) / sizeof(double) - 1;

@@ -109,10 +109,10 @@ constexpr KernelVariant kernel_variant(int form, int v) {
 // S_h2 algebraic 2.92 ms with 128-thread blocks, 2.70 with 64, 2.68 with 32;
 // 12,000 particles FP64 9.72 ms, 9.37, 9.58.  From 128 particles per SM on,
 // large blocks, whose warps share the fetched code: 30,000 particles FP64
-// 11.4 ms with 128 threads, 13.0 with 64.  There form 4 takes
-// one block of eight warps per SM with W_d in shared memory: 64 digesters
-// with 400,000 particles 115.9 ms (128 threads, W_d in registers) against
-// 83.1, 1M particles with slugs 34.0 against 27.1.
+// 11.4 ms with 128 threads, 13.0 with 64.  There form 4 takes one block of
+// eight warps per SM with W_d in shared memory: 64 digesters with 400,000
+// particles 115.9 ms (128 threads, W_d in registers) against 83.1, 1M
+// particles with slugs 34.0 against 27.1.
 constexpr int default_variant(int form, int64_t n, int sms) {
   return n <= (int64_t)64 * sms ? 5 : n <= (int64_t)128 * sms ? 3 : form == 4 ? 6 : 0;
 }

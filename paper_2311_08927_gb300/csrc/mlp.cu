@@ -44,16 +44,25 @@ __device__ __forceinline__ uint32_t pack2(__nv_bfloat16 lo, __nv_bfloat16 hi) {
   return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
 }
 
-// max((float)d, floor) with the conversion rounded to nearest even, on the
-// bit pattern: a hardware FP64 -> FP32 conversion occupies the FP64 pipe (one
-// warp instruction per 64 cycles and sub-partition), which 29 of them per
-// particle would make the bound of the features.  Below 2^-126 and for NaN
-// the floor, from 2^128 up infinity.
+// (float)d rounded to nearest even, on the bit pattern: a hardware FP64 ->
+// FP32 conversion occupies the FP64 pipe (one warp instruction per 64 cycles
+// and sub-partition), which 30 of them per particle would make the bound of
+// the features.  Below 2^-126 a signed zero; infinities and NaN as usual.
+__device__ __forceinline__ float narrow_rn(double d) {
+  const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+  const unsigned mag = hi & 0x7fffffffu, rest = lo << 3;
+  unsigned u = ((mag - 0x38000000u) << 3) | (lo >> 29);
+  u += rest > 0x80000000u || (rest == 0x80000000u && (u & 1u));
+  const bool nan = mag > 0x7ff00000u || (mag == 0x7ff00000u && lo != 0u);
+  u = mag < 0x38100000u ? 0u : mag >= 0x47f00000u ? (nan ? 0x7fc00000u : 0x7f800000u) : u;
+  return __uint_as_float(u | (hi & 0x80000000u));
+}
+// max((float)d, floor) in fewer operations: NaN and everything below 2^-126
+// give the floor.
 __device__ __forceinline__ float floored(double d) {
   const int hi = __double2hiint(d);
-  const unsigned lo = (unsigned)__double2loint(d);
+  const unsigned lo = (unsigned)__double2loint(d), rest = lo << 3;
   unsigned u = ((unsigned)(hi - 0x38000000) << 3) | (lo >> 29);
-  const unsigned rest = lo << 3;
   u += rest > 0x80000000u || (rest == 0x80000000u && (u & 1u));
   if (hi >= 0x47f00000) u = 0x7f800000u;
   const bool nan = hi >= 0x7ff00000 && !(hi == 0x7ff00000 && lo == 0u);
@@ -872,7 +881,8 @@ __device__ __forceinline__ void add_two_float(float& h, float& l, float x, float
 // FixedSum, where x^2 = p + e exactly with p the rounded square (p / 32 is
 // below 64 for log10 of any float); e is summed with its rounding errors.  1M samples: 470 us with one FP64 tree per
 // feature, 319 with FP64 joining trees in 4,880 CTAs, 154 with these in one
-// resident wave.  Bound by the logarithms' issue and latency.
+// resident wave, 112 with the next sample's values on their way and the
+// temperature narrowed by integers.  Bound by the logarithms' issue.
 constexpr int kGroup = 6;
 __global__ void __launch_bounds__(kThreads) feature_partials(const double* __restrict__ y,
                                                              int64_t ld,
@@ -884,13 +894,23 @@ __global__ void __launch_bounds__(kThreads) feature_partials(const double* __res
   float eh[kGroup], el[kGroup];
 #pragma unroll
   for (int j = 0; j < kGroup; ++j) eh[j] = el[j] = 0.0f;
-#pragma unroll 2
-  for (int64_t p = (int64_t)blockIdx.x * kThreads + threadIdx.x; p < n;
-       p += (int64_t)gridDim.x * kThreads) {
+  // each sample's values are fetched while the one before is worked on
+  const int64_t stride = (int64_t)gridDim.x * kThreads;
+  int64_t p = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+  double next[kGroup];
+  auto fetch = [&](int64_t q) {
+#pragma unroll
+    for (int j = 0; j < kGroup; ++j) next[j] = f0 + j < NS ? y[(int64_t)(f0 + j) * ld + q] : T[q];
+  };
+  if (p < n) fetch(p);
+  for (; p < n; p += stride) {
+    float x[kGroup];
+#pragma unroll
+    for (int j = 0; j < kGroup; ++j) x[j] = narrow_rn(next[j]);
+    if (p + stride < n) fetch(p + stride);
 #pragma unroll
     for (int j = 0; j < kGroup; ++j) {
-      const int f = f0 + j;
-      const float v = f < NS ? log10f(floored(y[(int64_t)f * ld + p])) : (float)T[p] * 0.01f;
+      const float v = f0 + j < NS ? log10f(fmaxf(x[j], kLogFloor)) : x[j] * 0.01f;
       a[j].add(v);
       const float sq = __fmul_rn(v, v), e = fmaf(v, v, -sq);
       b[j].add(sq * 0.03125f);
@@ -949,8 +969,8 @@ __global__ void __launch_bounds__(kThreads) moments_finish(const double* part, i
 
 // log10 of a positive normal double: x = 2^k m with m in [1/sqrt 2, sqrt 2),
 // log m = 2 atanh(s) = 2 (s + s^3/3 + s^5/5 + ..), s = (m - 1)/(m + 1), |s| <
-// 0.1716: the first term left out, s^23/23, is below 2e-19.  Some 20 FP64
-// instructions where the general function takes twice that.  Other arguments
+// 0.1716: the first term left out, s^23/23, is below 2e-19.  Some 16 FP64
+// instructions where the general function takes over twice that.  Other arguments
 // take the general function.
 __device__ __forceinline__ double log10_normal(double x) {
   const int hi = __double2hiint(x);
@@ -960,9 +980,14 @@ __device__ __forceinline__ double log10_normal(double x) {
   const double m = __hiloint2double(hi - (k << 20), __double2loint(x));
   const double s = (m - 1.0) * rcp<double>(m + 1.0);
   const double z = s * s;
-  double p = 1.0 / 21.0;
+  // the terms from s^13 on weigh less than 2^-34 of the sum: FP32
+  const float zf = cvt<float>(z);
+  float q = 1.0f / 21.0f;
 #pragma unroll
-  for (int i = 19; i >= 3; i -= 2) p = fma(p, z, 1.0 / i);
+  for (int i = 19; i >= 13; i -= 2) q = fmaf(q, zf, 1.0f / i);
+  double p = cvt<double>(q);
+#pragma unroll
+  for (int i = 11; i >= 3; i -= 2) p = fma(p, z, 1.0 / i);
   const double l = fma(s * z, p, s);  // atanh(s)
   // log10 2 in two parts, the first with 32 trailing zero bits: k times it is exact
   const double c1 = 0.30102992057800293, c2 = 7.508597826552624e-08;
@@ -972,8 +997,8 @@ __device__ __forceinline__ double log10_normal(double x) {
 
 // Partials of the two targets log10 S_H and log10 h: part[b][0][k],
 // part[b][1][k].  The logarithms, rounded to float, wait in Y for the
-// standardisation.  Bound by the FP64 pipe (some 50 instructions per sample):
-// 1M samples 140 us with the general logarithm, 100 here; the
+// standardisation.  Bound by the FP64 pipe (some 40 instructions per sample):
+// 1M samples 140 us with the general logarithm, 82 here; the
 // standardisation, which formed them anew, took 122 and takes 6.
 __global__ void __launch_bounds__(kThreads) target_partials(const double* __restrict__ SH,
                                                             const double* __restrict__ h,
@@ -987,8 +1012,8 @@ __global__ void __launch_bounds__(kThreads) target_partials(const double* __rest
     v[1] += t1;
     v[2] = fma(t0, t0, v[2]);
     v[3] = fma(t1, t1, v[3]);
-    Y[2 * p] = (float)t0;
-    Y[2 * p + 1] = (float)t1;
+    Y[2 * p] = narrow_rn(t0);
+    Y[2 * p + 1] = narrow_rn(t1);
   }
   block_sums<4>(v, s, part + (int64_t)blockIdx.x * 4, 1);
 }
@@ -1243,7 +1268,7 @@ chad_status chad_mlp_feature_norm(const double* y, int64_t ld, const double* T, 
   if (n < 2 || !y || !T || !norm || !scratch || ld < n) return CHAD_E_INVALID;
   if (scratch_bytes < chad_mlp_prep_scratch_bytes()) return CHAD_E_INVALID;
   cudaStream_t s = (cudaStream_t)stream;
-  const int nb = mlp::prep::grid_for(n, mlp::sm_count() * 7 / 5);
+  const int nb = mlp::prep::grid_for(n, mlp::sm_count());
   double* part = static_cast<double*>(scratch);
   mlp::prep::feature_partials<<<dim3(nb, mlp::prep::kNF / mlp::prep::kGroup), mlp::prep::kThreads, 0, s>>>(y, ld, T, n, part);
   // padding features: mean 0, 1/std 1
