@@ -14,6 +14,7 @@
 #include <cmath>
 #include <cstdint>
 #include <cstring>
+#include <type_traits>
 
 #include "model.h"
 
@@ -512,18 +513,25 @@ CHAD_HD void hill(R S, R invK, R n, int ni, R& I, R& dI) {
 // with P >= 0: E decreases in S and the root is unique.
 template <class F>
 struct H2Bal {
-  F C0, PKfa, PKc4, PKpro, Ph2, kD, Kfa, Kc4, Kpro, Kh2;  // PK = P K
+  F C0, Pfa, Pc4, Ppro, Ph2, kD, Kfa, Kc4, Kpro, Kh2;  // Pfa, Pc4, Ppro: times their K in FP64
 };
 
 // Factors of the rates that do not hold S_h2 (Eq. 3-6 inhibitions and Monod
 // terms): formed once per evaluation point and shared by the Eq. 8 balance
 // and the rates, ten reciprocals and about 60 operations fewer than forming
-// them in both.  B5 and B12 carry the Arrhenius factor.  The FP64 forms are
+// them in both.  In FP64, B5 and B12 carry the Arrhenius factor (one product
+// instead of one per rate constant).  FP32 products keep the association that
+// they have had: the mixed forms' error estimates, and with them the choice
+// of a step, hang on the last bits of the FP32 rates.  The FP64 forms are
 // bound by the FP64 pipe, one warp instruction per 64 cycles and
 // sub-partition, so each instruction saved counts: with the partials below
 // and the products of structural zeros left out, 100,000 particles in the
 // shared-headspace cylinder take 54.5 ms instead of 58.0, ten fixed substeps
 // of 111,000 particles 8.54 instead of 9.18.
+template <class R>
+constexpr bool is_f32() {
+  return std::is_same<R, float>::value;
+}
 template <class R>
 struct Factors {
   R Ipaa, dIpaa, Iph2, dIph2;  // pH inhibitions (the aa form also of su, fa, c4, pro)
@@ -556,7 +564,7 @@ CHAD_HD void factors(const DC& c, const PQ& q, const Y* y, const AcidBase& ab, F
   k.rden = rcp<R>(S_bu + S_va + R(kC4Guard));
   k.gva = S_va * k.rden;
   k.gbu = S_bu * k.rden;
-  const R aN = R(q.arr) * k.IIN;
+  const R aN = is_f32<R>() ? k.IIN : R(q.arr) * k.IIN;
   k.B5 = k.Ipaa * aN;
   k.B12 = k.Iph2 * aN;
 }
@@ -566,14 +574,25 @@ CHAD_HD void h2_coeffs(const DC& c, const PQ& q, const Y* y, F D, const Factors<
                        H2Bal<F>& e) {
   const F kLa = F(c.k_La);
   const F KH2 = F(q.K_H_h2) * F(q.RT);
-  const F r4 = F(c.k_m_su) * F(y[iX_su]) * k.msu;
-  const F r5 = F(c.k_m_aa) * F(y[iX_aa]) * k.maa;
-  e.C0 = D * F(c.y_in[iS_h2]) + (F(c.su_h2) * r4 + F(c.aa_h2) * r5) * k.B5 + kLa * KH2 * F(y[iG_h2]);
-  e.PKfa = F(c.fa_h2) * (F(c.k_m_fa) * F(y[iX_fa]) * k.mfa) * k.B5 * F(c.K_I_h2_fa);
-  e.PKc4 = (F(c.va_h2) * (k.mva * k.gva) + F(c.bu_h2) * (k.mbu * k.gbu)) *
-           (F(c.k_m_c4) * F(y[iX_c4])) * k.B5 * F(c.K_I_h2_c4);
-  e.PKpro = F(c.pro_h2) * (F(c.k_m_pro) * F(y[iX_pro]) * k.mpo) * k.B5 * F(c.K_I_h2_pro);
-  e.Ph2 = F(c.k_m_h2) * F(y[iX_h2]) * k.B12;
+  if constexpr (is_f32<F>()) {
+    const F a = F(q.arr);
+    const F r4 = F(c.k_m_su) * a * F(y[iX_su]) * k.msu * k.B5;
+    const F r5 = F(c.k_m_aa) * a * F(y[iX_aa]) * k.maa * k.B5;
+    e.C0 = D * F(c.y_in[iS_h2]) + F(c.su_h2) * r4 + F(c.aa_h2) * r5 + kLa * KH2 * F(y[iG_h2]);
+    e.Pfa = F(c.fa_h2) * F(c.k_m_fa) * a * F(y[iX_fa]) * k.mfa * k.B5;
+    e.Pc4 = (F(c.va_h2) * k.mva * k.gva + F(c.bu_h2) * k.mbu * k.gbu) * F(c.k_m_c4) * a * F(y[iX_c4]) * k.B5;
+    e.Ppro = F(c.pro_h2) * F(c.k_m_pro) * a * F(y[iX_pro]) * k.mpo * k.B5;
+    e.Ph2 = F(c.k_m_h2) * a * F(y[iX_h2]) * k.B12;
+  } else {
+    const F r4 = F(c.k_m_su) * F(y[iX_su]) * k.msu;
+    const F r5 = F(c.k_m_aa) * F(y[iX_aa]) * k.maa;
+    e.C0 = D * F(c.y_in[iS_h2]) + (F(c.su_h2) * r4 + F(c.aa_h2) * r5) * k.B5 + kLa * KH2 * F(y[iG_h2]);
+    e.Pfa = F(c.fa_h2) * (F(c.k_m_fa) * F(y[iX_fa]) * k.mfa) * k.B5 * F(c.K_I_h2_fa);
+    e.Pc4 = (F(c.va_h2) * (k.mva * k.gva) + F(c.bu_h2) * (k.mbu * k.gbu)) *
+            (F(c.k_m_c4) * F(y[iX_c4])) * k.B5 * F(c.K_I_h2_c4);
+    e.Ppro = F(c.pro_h2) * (F(c.k_m_pro) * F(y[iX_pro]) * k.mpo) * k.B5 * F(c.K_I_h2_pro);
+    e.Ph2 = F(c.k_m_h2) * F(y[iX_h2]) * k.B12;
+  }
   e.kD = kLa + D;
   e.Kfa = F(c.K_I_h2_fa);
   e.Kc4 = F(c.K_I_h2_c4);
@@ -581,13 +600,19 @@ CHAD_HD void h2_coeffs(const DC& c, const PQ& q, const Y* y, F D, const Factors<
   e.Kh2 = F(c.K_S_h2);
 }
 
-// E(S) and dE/dS of Eq. 8 from the coefficients; h (may be null) receives
-// E''/2.
+// E(S) and dE/dS of Eq. 8 from the coefficients; h (may be null; FP64)
+// receives E''/2.
 template <class F>
 CHAD_HD F h2_eval(const H2Bal<F>& e, F S, F& dE, F* h = nullptr) {
   const F rfa = rcp<F>(e.Kfa + S), rc4 = rcp<F>(e.Kc4 + S), rpr = rcp<F>(e.Kpro + S);
   const F rh = rcp<F>(e.Kh2 + S);
-  const F tfa = e.PKfa * rfa, tc4 = e.PKc4 * rc4, tpr = e.PKpro * rpr, th = e.Ph2 * rh;
+  if constexpr (is_f32<F>()) {
+    const F Ifa = e.Kfa * rfa, Ic4 = e.Kc4 * rc4, Ipr = e.Kpro * rpr;
+    dE = F(0) - (e.Pfa * Ifa * rfa + e.Pc4 * Ic4 * rc4 + e.Ppro * Ipr * rpr +
+                 e.Ph2 * e.Kh2 * rh * rh + e.kD);
+    return e.C0 + e.Pfa * Ifa + e.Pc4 * Ic4 + e.Ppro * Ipr - e.Ph2 * S * rh - e.kD * S;
+  }
+  const F tfa = e.Pfa * rfa, tc4 = e.Pc4 * rc4, tpr = e.Ppro * rpr, th = e.Ph2 * rh;
   const F dfa = tfa * rfa, dc4 = tc4 * rc4, dpr = tpr * rpr, dh = th * (e.Kh2 * rh);
   dE = F(0) - (dfa + dc4 + dpr + dh + e.kD);
   if (h) *h = dfa * rfa + dc4 * rc4 + dpr * rpr + dh * rh;
@@ -683,12 +708,18 @@ CHAD_HD void rates(const DC& c, const PQ& q, const R* y, const AcidBase& ab, con
   const R rac = rcp<R>(R(c.K_S_ac) + y[iS_ac]), rh2 = rcp<R>(R(c.K_S_h2) + S_h2);
   const R mac = y[iS_ac] * rac, mh2 = S_h2 * rh2;
   const R B7 = k.B5 * Ih2fa, B8 = k.B5 * Ih2c4, B10 = k.B5 * Ih2pro;
-  const R B11 = Ipac * (a * k.IIN) * Inh3;
-  const R A5 = R(c.k_m_su) * y[iX_su], A6 = R(c.k_m_aa) * y[iX_aa], A7 = R(c.k_m_fa) * y[iX_fa];
-  const R A8 = R(c.k_m_c4) * y[iX_c4], A10 = R(c.k_m_pro) * y[iX_pro], A11 = R(c.k_m_ac) * y[iX_ac];
-  const R A12 = R(c.k_m_h2) * y[iX_h2];
+  // the Arrhenius factor: in the rate constants (FP32) or in the B (FP64)
+  const R aK = is_f32<R>() ? a : R(1), aB = is_f32<R>() ? R(1) : a;
+  const R B11 = Ipac * (aB * k.IIN) * Inh3;
+  const R ksu = R(c.k_m_su) * aK, kaa = R(c.k_m_aa) * aK, kfa = R(c.k_m_fa) * aK,
+          kc4 = R(c.k_m_c4) * aK, kpo = R(c.k_m_pro) * aK, kac = R(c.k_m_ac) * aK,
+          kh2 = R(c.k_m_h2) * aK;
+  const R A5 = ksu * y[iX_su], A6 = kaa * y[iX_aa], A7 = kfa * y[iX_fa], A8 = kc4 * y[iX_c4];
+  const R A10 = kpo * y[iX_pro], A11 = kac * y[iX_ac], A12 = kh2 * y[iX_h2];
   const R tva = k.mva * k.gva, tbu = k.mbu * k.gbu;
-  const R p5 = A5 * k.msu, p6 = A6 * k.maa, p7 = A7 * k.mfa, p8 = A8 * tva, p9 = A8 * tbu;
+  const R p5 = A5 * k.msu, p6 = A6 * k.maa, p7 = A7 * k.mfa;
+  const R p8 = is_f32<R>() ? A8 * k.mva * k.gva : A8 * tva;
+  const R p9 = is_f32<R>() ? A8 * k.mbu * k.gbu : A8 * tbu;
   const R p10 = A10 * k.mpo, p11 = A11 * mac, p12 = A12 * mh2;
   o.r[4] = p5 * k.B5;
   o.r[5] = p6 * k.B5;
@@ -718,7 +749,71 @@ CHAD_HD void rates(const DC& c, const PQ& q, const R* y, const AcidBase& ab, con
   o.r[20] = kLa * (y[iS_ch4] - KCH4 * y[iG_ch4]);
   o.r[21] = kLa * (y[iS_IC] * fco2 - KCO2 * y[iG_co2]);
 
-  if (J) {
+  if constexpr (J && is_f32<R>()) {
+    // FP32 partials (sc is 1 here), each product associated from the left
+    const R dIIN = R(c.K_S_IN) * k.rIN * k.rIN;
+    o.d1 = kdis; o.d2 = kch; o.d3 = kpr; o.d4 = kli;
+    // rho5: S_su, X_su, S_IN
+    o.d5[0] = A5 * (R(c.K_S_su) * k.rsu * k.rsu) * k.B5;
+    o.d5[1] = ksu * k.msu * k.B5;
+    o.d5[2] = A5 * k.msu * k.Ipaa * dIIN;
+    o.s5 = A5 * k.msu * k.dIpaa * k.IIN;
+    // rho6: S_aa, X_aa, S_IN
+    o.d6[0] = A6 * (R(c.K_S_aa) * k.raa * k.raa) * k.B5;
+    o.d6[1] = kaa * k.maa * k.B5;
+    o.d6[2] = A6 * k.maa * k.Ipaa * dIIN;
+    o.s6 = A6 * k.maa * k.dIpaa * k.IIN;
+    // rho7: S_fa, X_fa, S_IN, S_h2
+    o.d7[0] = A7 * (R(c.K_S_fa) * k.rfs * k.rfs) * B7;
+    o.d7[1] = kfa * k.mfa * B7;
+    o.d7[2] = A7 * k.mfa * k.Ipaa * dIIN * Ih2fa;
+    o.d7[3] = -A7 * k.mfa * k.B5 * Ih2fa * rfa;   // dI/dS_h2 = -K/(K+S)^2 = -I r
+    o.s7 = A7 * k.mfa * k.dIpaa * k.IIN * Ih2fa;
+    // rho8, rho9: S_va, S_bu, X_c4, S_IN, S_h2
+    const R rd2 = k.rden * k.rden;
+    const R dgva_va = (y[iS_bu] + R(kC4Guard)) * rd2, dgva_bu = -y[iS_va] * rd2;
+    const R dgbu_bu = (y[iS_va] + R(kC4Guard)) * rd2, dgbu_va = -y[iS_bu] * rd2;
+    const R dmva = R(c.K_S_c4) * k.rva * k.rva, dmbu = R(c.K_S_c4) * k.rbu * k.rbu;
+    o.d8[0] = A8 * B8 * (dmva * k.gva + k.mva * dgva_va);
+    o.d8[1] = A8 * B8 * k.mva * dgva_bu;
+    o.d8[2] = kc4 * k.mva * k.gva * B8;
+    o.d8[3] = A8 * k.mva * k.gva * k.Ipaa * dIIN * Ih2c4;
+    o.d8[4] = -A8 * k.mva * k.gva * k.B5 * Ih2c4 * rc4;
+    o.s8 = A8 * k.mva * k.gva * k.dIpaa * k.IIN * Ih2c4;
+    o.d9[0] = A8 * B8 * k.mbu * dgbu_va;
+    o.d9[1] = A8 * B8 * (dmbu * k.gbu + k.mbu * dgbu_bu);
+    o.d9[2] = kc4 * k.mbu * k.gbu * B8;
+    o.d9[3] = A8 * k.mbu * k.gbu * k.Ipaa * dIIN * Ih2c4;
+    o.d9[4] = -A8 * k.mbu * k.gbu * k.B5 * Ih2c4 * rc4;
+    o.s9 = A8 * k.mbu * k.gbu * k.dIpaa * k.IIN * Ih2c4;
+    // rho10: S_pro, X_pro, S_IN, S_h2
+    o.d10[0] = A10 * (R(c.K_S_pro) * k.rpo * k.rpo) * B10;
+    o.d10[1] = kpo * k.mpo * B10;
+    o.d10[2] = A10 * k.mpo * k.Ipaa * dIIN * Ih2pro;
+    o.d10[3] = -A10 * k.mpo * k.B5 * Ih2pro * rpr;
+    o.s10 = A10 * k.mpo * k.dIpaa * k.IIN * Ih2pro;
+    // rho11: S_ac, X_ac, S_IN (I_IN and free ammonia)
+    const R dInh3 = -Inh3 * rnh;  // dI_nh3 / dS_nh3
+    o.d11[0] = A11 * (R(c.K_S_ac) * rac * rac) * B11;
+    o.d11[1] = kac * mac * B11;
+    o.d11[2] = A11 * mac * Ipac * (dIIN * Inh3 + k.IIN * dInh3 * r_nh3);
+    o.s11 = A11 * mac * k.IIN * (dIpac * Inh3 - Ipac * dInh3 * nh3 * R(ab.r_IN));
+    // rho12: S_h2, X_h2, S_IN
+    o.d12[0] = A12 * (R(c.K_S_h2) * rh2 * rh2) * k.B12;
+    o.d12[1] = kh2 * mh2 * k.B12;
+    o.d12[2] = A12 * mh2 * k.Iph2 * dIIN;
+    o.s12 = A12 * mh2 * k.dIph2 * k.IIN;
+#pragma unroll
+    for (int i = 0; i < 7; ++i) o.ddec[i] = kd[i];
+    // transfers
+    o.dT8[0] = kLa; o.dT8[1] = -kLa * KH2;
+    o.dT9[0] = kLa; o.dT9[1] = -kLa * KCH4;
+    o.dT10[0] = kLa * fco2; o.dT10[1] = -kLa * KCO2;
+    o.sT10 = kLa * y[iS_IC] * R(q.K_a_co2) * rco2 * rco2;
+    o.qvs = o.qv;
+    o.dqv = kpv * (R(2) * P - R(c.P_atm)) * invPa;
+    o.P_h2 = P_h2; o.P_ch4 = P_ch4; o.P_co2 = P_co2;
+  } else if constexpr (J) {
     o.d1 = kdis * sc; o.d2 = kch * sc; o.d3 = kpr * sc; o.d4 = kli * sc;
     // scaled factors of the uptakes and their derivatives to S_IN (G) and S_H (H)
     const R as = a * sc, aN = as * k.IIN;
@@ -726,18 +821,18 @@ CHAD_HD void rates(const DC& c, const PQ& q, const R* y, const AcidBase& ab, con
     const R Bs = k.B5 * sc, G = k.Ipaa * dIIN, H = k.dIpaa * aN;
     // rho5: S_su, X_su, S_IN
     o.d5[0] = A5 * Bs * (R(c.K_S_su) * k.rsu * k.rsu);
-    o.d5[1] = R(c.k_m_su) * k.msu * Bs;
+    o.d5[1] = ksu * k.msu * Bs;
     o.d5[2] = p5 * G;
     o.s5 = p5 * H;
     // rho6: S_aa, X_aa, S_IN
     o.d6[0] = A6 * Bs * (R(c.K_S_aa) * k.raa * k.raa);
-    o.d6[1] = R(c.k_m_aa) * k.maa * Bs;
+    o.d6[1] = kaa * k.maa * Bs;
     o.d6[2] = p6 * G;
     o.s6 = p6 * H;
     // rho7: S_fa, X_fa, S_IN, S_h2 (dI/dS_h2 = -K/(K+S)^2 = -I r)
     const R Bs7 = Bs * Ih2fa, p7i = p7 * Ih2fa;
     o.d7[0] = A7 * Bs7 * (R(c.K_S_fa) * k.rfs * k.rfs);
-    o.d7[1] = R(c.k_m_fa) * k.mfa * Bs7;
+    o.d7[1] = kfa * k.mfa * Bs7;
     o.d7[2] = p7i * G;
     o.d7[3] = -p7i * Bs * rfa;
     o.s7 = p7i * H;
@@ -746,7 +841,7 @@ CHAD_HD void rates(const DC& c, const PQ& q, const R* y, const AcidBase& ab, con
     const R dgva_va = (y[iS_bu] + R(kC4Guard)) * rd2, dgva_bu = -y[iS_va] * rd2;
     const R dgbu_bu = (y[iS_va] + R(kC4Guard)) * rd2, dgbu_va = -y[iS_bu] * rd2;
     const R dmva = R(c.K_S_c4) * k.rva * k.rva, dmbu = R(c.K_S_c4) * k.rbu * k.rbu;
-    const R Bs8 = Bs * Ih2c4, AB8 = A8 * Bs8, kB8 = R(c.k_m_c4) * Bs8, Bsr = Bs * rc4;
+    const R Bs8 = Bs * Ih2c4, AB8 = A8 * Bs8, kB8 = kc4 * Bs8, Bsr = Bs * rc4;
     const R p8i = p8 * Ih2c4, p9i = p9 * Ih2c4;
     o.d8[0] = AB8 * (dmva * k.gva + k.mva * dgva_va);
     o.d8[1] = AB8 * (k.mva * dgva_bu);
@@ -763,7 +858,7 @@ CHAD_HD void rates(const DC& c, const PQ& q, const R* y, const AcidBase& ab, con
     // rho10: S_pro, X_pro, S_IN, S_h2
     const R Bs10 = Bs * Ih2pro, p10i = p10 * Ih2pro;
     o.d10[0] = A10 * Bs10 * (R(c.K_S_pro) * k.rpo * k.rpo);
-    o.d10[1] = R(c.k_m_pro) * k.mpo * Bs10;
+    o.d10[1] = kpo * k.mpo * Bs10;
     o.d10[2] = p10i * G;
     o.d10[3] = -p10i * Bs * rpr;
     o.s10 = p10i * H;
@@ -771,13 +866,13 @@ CHAD_HD void rates(const DC& c, const PQ& q, const R* y, const AcidBase& ab, con
     const R dInh3 = -Inh3 * rnh;  // dI_nh3 / dS_nh3
     const R Bs11 = B11 * sc;
     o.d11[0] = A11 * Bs11 * (R(c.K_S_ac) * rac * rac);
-    o.d11[1] = R(c.k_m_ac) * mac * Bs11;
+    o.d11[1] = kac * mac * Bs11;
     o.d11[2] = p11 * (Ipac * (dIIN * Inh3 + aN * (dInh3 * r_nh3)));
     o.s11 = p11 * (aN * (dIpac * Inh3 - Ipac * dInh3 * nh3 * R(ab.r_IN)));
     // rho12: S_h2, X_h2, S_IN
     const R Bs12 = k.B12 * sc;
     o.d12[0] = A12 * Bs12 * (R(c.K_S_h2) * rh2 * rh2);
-    o.d12[1] = R(c.k_m_h2) * mh2 * Bs12;
+    o.d12[1] = kh2 * mh2 * Bs12;
     o.d12[2] = p12 * (k.Iph2 * dIIN);
     o.s12 = p12 * (k.dIph2 * aN);
 #pragma unroll

@@ -772,8 +772,7 @@ __global__ void __launch_bounds__(BS, MINB) integrate_kernel(StepArgs a) {
         // high words, a few 1e-6 relative), its error and magnitude kept in
         // FP64 and the norm formed from them: a near tie can pick a ratio
         // 4e-6 below the largest.  Comparing 29 ratios in FP64 took five
-        // slots of the FP64 pipe per species.  Not finite -> the ratio is
-        // infinite and stays the largest.
+        // slots of the FP64 pipe per species.  Not finite: an infinite norm.
         double en = 0.0, ym = 0.0, at = 1.0;
         float best = 0.0f;
         const float rtol = cvt<float>(a.rtol);
@@ -792,7 +791,7 @@ __global__ void __launch_bounds__(BS, MINB) integrate_kernel(StepArgs a) {
           }
         }
         const double sn = fma(a.rtol, fabs(ym), at);
-        norm = fabs(en) * rcp<double>(sn) * (hh * (1.0 / 6.0));
+        norm = best == INFINITY ? NR(INFINITY) : fabs(en) * rcp<double>(sn) * (hh * (1.0 / 6.0));
       } else {
         float nf = 0.0f;
         const float rtol = cvt<float>(a.rtol);

@@ -480,7 +480,7 @@ struct Pipe {
   __nv_bfloat16 B12[TILE * kB12];  // A1 0-63, X 64-95, ones 96, zeros 97-111
   __nv_bfloat16 A3[TILE * kW3];    // A2 0-63, ones 64, zeros 65-71
   __nv_bfloat16 B3[TILE * kB3];    // dO 0-1, zeros 2-15
-  float2 part[2][TILE];            // the two halves of the output layer's sums
+  float2 part[2][TILE];            // the output layer's sums after each half of the units
 };
 
 struct Smem {
@@ -626,8 +626,7 @@ __global__ void __launch_bounds__(kThreads, 1) grad_kernel(const __nv_bfloat16* 
     }
     if (!wait()) break;
     // A2 and the output layer's half sums, silu' kept
-    float ds2[HID / 2];
-    float o0 = 0.0f, o1 = 0.0f;
+    float ds2[HID / 2], a2[HID / 2];
 #pragma unroll
     for (int c = 0; c < HID / 2; c += 16) {
       float z[16];
@@ -638,19 +637,34 @@ __global__ void __launch_bounds__(kThreads, 1) grad_kernel(const __nv_bfloat16* 
         const float sg = sigmoid(zz);
         ds2[c + j] = sg * (1.0f + zz * (1.0f - sg));
         z[j] = __bfloat162float(__float2bfloat16_rn(zz * sg));
-        o0 = fmaf(z[j], s.W3[u0 + c + j], o0);
-        o1 = fmaf(z[j], s.W3[HID + u0 + c + j], o1);
+        a2[c + j] = z[j];
       }
       *reinterpret_cast<uint4*>(&b.A3[kmaj(r, u0 + c, kW3)]) = pack8(z);
       *reinterpret_cast<uint4*>(&b.A3[kmaj(r, u0 + c + 8, kW3)]) = pack8(z + 8);
     }
-    b.part[half][r] = make_float2(o0, o1);
+    // the sums run over the units in order, the second half continuing the
+    // first's: dO is rounded to BF16, which a sum in two parts would shift
+    // now and then by a last place
+    float2 o = make_float2(s.b3[0], s.b3[1]);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if (h == 1) pipe_bar(bar_id);
+      if (half == h) {
+        if (h == 1) o = b.part[0][r];
+#pragma unroll
+        for (int c = 0; c < HID / 2; ++c) {
+          o.x = fmaf(a2[c], s.W3[u0 + c], o.x);
+          o.y = fmaf(a2[c], s.W3[HID + u0 + c], o.y);
+        }
+        b.part[h][r] = o;
+      }
+    }
     pipe_bar(bar_id);
-    const float2 h0 = b.part[0][r], h1 = b.part[1][r];
+    o = b.part[1][r];
     float d0 = 0.0f, d1 = 0.0f;
     if (live) {
-      d0 = (s.b3[0] + h0.x) + h1.x - y0;
-      d1 = (s.b3[1] + h0.y) + h1.y - y1;
+      d0 = o.x - y0;
+      d1 = o.y - y1;
       if (half == 0) lsum += (d0 * d0 + d1 * d1) * inv_n;
       d0 *= 2.0f * inv_n;
       d1 *= 2.0f * inv_n;
@@ -839,10 +853,11 @@ __device__ __forceinline__ void block_sums(double (&v)[K], double* s, double* ou
 
 // Exact sums of floats without the FP64 pipe (an FP64 addition holds it for
 // 64 cycles per warp).  A value |x| < 64 is added to a 64-bit integer in
-// units of 2^-38, in two pieces that adding 1.5 x 2^23 rounds to integers;
-// every float of magnitude 2^-14 or more is a multiple of that unit, so the
-// sum is exact but for smaller terms, each rounded by at most 2^-39.  Room
-// for 2^63-38 / 64 = 524,288 terms.  Values from 64 up and NaN go to `out`.
+// units of 2^-36, in two pieces that adding 1.5 x 2^23 rounds to integers;
+// every float of magnitude 2^-12 or more is a multiple of that unit, so the
+// sum is exact but for smaller terms, each rounded by at most 2^-37.  Room
+// for 2^63-36 / 64 = 2^21 terms of the largest size in a warp, that is for
+// more samples than the device holds.  Values from 64 up and NaN go to `out`.
 struct FixedSum {
   long long q = 0;
   float out = 0.0f;
@@ -859,12 +874,12 @@ struct FixedSum {
     const bool in = fabsf(x) < 64.0f;
     const float t = in ? x * 65536.0f : 0.0f;
     const float h = t + M;
-    const float l = (t - (h - M)) * 4194304.0f + M;
-    q += (long long)(__float_as_int(h) - 0x4b400000) * 4194304ll + (__float_as_int(l) - 0x4b400000);
+    const float l = (t - (h - M)) * 1048576.0f + M;
+    q += (long long)(__float_as_int(h) - 0x4b400000) * 1048576ll + (__float_as_int(l) - 0x4b400000);
     if (!in) out += x;
   }
   __device__ __forceinline__ double value() const {
-    return (double)q * 3.637978807091713e-12 + (double)out;  // 2^-38
+    return (double)q * 1.4551915228366852e-11 + (double)out;  // 2^-36
   }
 };
 
