@@ -426,7 +426,8 @@ chad_status chad_load_particles(chad_ctx* c, int digester, int64_t n, const doub
     if (pos) {
       CK(c, copy_rows(c->d_pos + o, c->ld, pos, n, n, 3, k, s), "load pos");
     } else {
-      CK(c, cudaMemset2DAsync(c->d_pos + o, sizeof(double) * c->ld, 0, sizeof(double) * n, 3, s), "zero pos");
+      for (int i = 0; i < 3; ++i)
+        CK(c, cudaMemsetAsync(c->d_pos + (size_t)i * c->ld + o, 0, sizeof(double) * n, s), "zero pos");
     }
     auto fill = [&](double* dst, const double* src, double dflt) -> cudaError_t {
       if (src) return cudaMemcpyAsync(dst + o, src, sizeof(double) * n, k, s);

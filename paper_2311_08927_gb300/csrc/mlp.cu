@@ -454,7 +454,8 @@ constexpr size_t smem_bytes() { return sizeof(Smem) + 128; }
 // The tensor cores are a few per cent busy: a tile's time is its chain of
 // epilogues.  So
 //   * two threads share a sample, each with half of the hidden units (the two
-//     warps of a lane quarter), and meet once, for the output layer;
+//     warps of a lane quarter), and meet for the output layer, whose sums the
+//     second half continues from the first's (the order of one thread's sum);
 //   * one sigmoid per pre-activation serves SiLU and its derivative, which
 //     waits in registers for the backward pass;
 //   * every activation is stored once, as 16-byte vectors in (sample, unit)
