@@ -852,35 +852,31 @@ __device__ __forceinline__ void block_sums(double (&v)[K], double* s, double* ou
   __syncthreads();
 }
 
-// Exact sums of floats without the FP64 pipe (an FP64 addition holds it for
-// 64 cycles per warp).  A value |x| < 64 is added to a 64-bit integer in
-// units of 2^-36, in two pieces that adding 1.5 x 2^23 rounds to integers;
-// every float of magnitude 2^-12 or more is a multiple of that unit, so the
-// sum is exact but for smaller terms, each rounded by at most 2^-37.  Room
-// for 2^63-36 / 64 = 2^21 terms of the largest size in a warp, that is for
-// more samples than the device holds.  Values from 64 up and NaN go to `out`.
+// Sums of floats without the FP64 pipe (an FP64 addition holds it for 64
+// cycles per warp).  A value |x| < 64 is added to a 64-bit integer in units of
+// 2^-36, in two pieces that adding 1.5 x 2^23 rounds to integers; add returns
+// what the rounding left out, exactly (zero from |x| = 2^-12 up, whose floats
+// are multiples of the unit, at most 2^-37 below).  Room for 2^63-36 / 64 =
+// 2^21 terms of the largest size in a warp, that is for more samples than the
+// device holds.
 struct FixedSum {
   long long q = 0;
-  float out = 0.0f;
   // the sum over the warp's lanes, in every lane
   __device__ __forceinline__ void warp_sum() {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      q += __shfl_xor_sync(0xffffffffu, q, o);
-      out += __shfl_xor_sync(0xffffffffu, out, o);
-    }
+    for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
   }
-  __device__ __forceinline__ void add(float x) {
+  __device__ __forceinline__ float add(float x) {
     const float M = 12582912.0f;
-    const bool in = fabsf(x) < 64.0f;
-    const float t = in ? x * 65536.0f : 0.0f;
+    const float t = x * 65536.0f;
     const float h = t + M;
-    const float l = (t - (h - M)) * 1048576.0f + M;
+    const float s = (t - (h - M)) * 1048576.0f;
+    const float l = s + M;
     q += (long long)(__float_as_int(h) - 0x4b400000) * 1048576ll + (__float_as_int(l) - 0x4b400000);
-    if (!in) out += x;
+    return (s - (l - M)) * 1.4551915228366852e-11f;  // 2^-36
   }
   __device__ __forceinline__ double value() const {
-    return (double)q * 1.4551915228366852e-11 + (double)out;  // 2^-36
+    return (double)q * 1.4551915228366852e-11;
   }
 };
 
@@ -895,10 +891,13 @@ __device__ __forceinline__ void add_two_float(float& h, float& l, float x, float
 // grid-stride share of the samples: part[b][0][f], part[b][1][f], each thread
 // with the sums of six features in registers (blockIdx.y).  x and p go through
 // FixedSum, where x^2 = p + e exactly with p the rounded square (p / 32 is
-// below 64 for log10 of any float); e is summed with its rounding errors.  1M samples: 470 us with one FP64 tree per
-// feature, 319 with FP64 joining trees in 4,880 CTAs, 154 with these in one
-// resident wave, 112 with the next sample's values on their way and the
-// temperature narrowed by integers.  Bound by the logarithms' issue.
+// below 64 for |x| < 45, that is for log10 of any float); e and what FixedSum
+// leaves out of p are summed in two floats, what it leaves out of x in one.
+// The variance of a (nearly) constant feature is the difference of two sums
+// that agree to their last digits: without the part left out, a feature of
+// y = 0.87 with no spread (x^2 = 0.004, 2^-31 per unit) got a standard
+// deviation of 1.5e-5.  1M samples: 470 us with one FP64 tree per feature,
+// 112 here.  Bound by the logarithms' issue.
 constexpr int kGroup = 6;
 __global__ void __launch_bounds__(kThreads) feature_partials(const double* __restrict__ y,
                                                              int64_t ld,
@@ -907,9 +906,10 @@ __global__ void __launch_bounds__(kThreads) feature_partials(const double* __res
   __shared__ double s[2][kThreads / 32][kGroup];
   const int f0 = blockIdx.y * kGroup;
   FixedSum a[kGroup], b[kGroup];
-  float eh[kGroup], el[kGroup];
+  float la[kGroup], eh[kGroup], el[kGroup];  // left out of a; the rest of b
+  double hot[2] = {0.0, 0.0};                // temperatures from 4,500 K up
 #pragma unroll
-  for (int j = 0; j < kGroup; ++j) eh[j] = el[j] = 0.0f;
+  for (int j = 0; j < kGroup; ++j) la[j] = eh[j] = el[j] = 0.0f;
   // each sample's values are fetched while the one before is worked on
   const int64_t stride = (int64_t)gridDim.x * kThreads;
   int64_t p = (int64_t)blockIdx.x * kThreads + threadIdx.x;
@@ -927,10 +927,20 @@ __global__ void __launch_bounds__(kThreads) feature_partials(const double* __res
 #pragma unroll
     for (int j = 0; j < kGroup; ++j) {
       const float v = f0 + j < NS ? log10f(fmaxf(x[j], kLogFloor)) : x[j] * 0.01f;
-      a[j].add(v);
-      const float sq = __fmul_rn(v, v), e = fmaf(v, v, -sq);
-      b[j].add(sq * 0.03125f);
-      add_two_float(eh[j], el[j], e, 0.0f);
+      const bool in = fabsf(v) < 45.0f;
+      const float w = in ? v : 0.0f;
+      const float ra = a[j].add(w);
+      if (j == kGroup - 1 && f0 + j == NS) {
+        la[j] += ra;
+        if (!in) {
+          hot[0] += v;
+          hot[1] += (double)v * v;
+        }
+      } else {
+        la[j] += in ? ra : v;  // the logarithm of an infinite state
+      }
+      const float sq = __fmul_rn(w, w), e = fmaf(w, w, -sq);
+      add_two_float(eh[j], el[j], e + 32.0f * b[j].add(sq * 0.03125f), 0.0f);
     }
   }
   // the joining trees stay off the FP64 pipe too: integers and TwoSums
@@ -939,12 +949,22 @@ __global__ void __launch_bounds__(kThreads) feature_partials(const double* __res
     a[j].warp_sum();
     b[j].warp_sum();
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
+    for (int o = 16; o > 0; o >>= 1) {
+      la[j] += __shfl_xor_sync(0xffffffffu, la[j], o);
       add_two_float(eh[j], el[j], __shfl_xor_sync(0xffffffffu, eh[j], o),
                     __shfl_xor_sync(0xffffffffu, el[j], o));
+    }
     if ((threadIdx.x & 31) == 0) {
-      s[0][threadIdx.x >> 5][j] = a[j].value();
+      s[0][threadIdx.x >> 5][j] = a[j].value() + (double)la[j];
       s[1][threadIdx.x >> 5][j] = 32.0 * b[j].value() + ((double)eh[j] + (double)el[j]);
+    }
+  }
+  if (__any_sync(0xffffffffu, __double_as_longlong(hot[0]) != 0)) {
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) hot[k] += __shfl_xor_sync(0xffffffffu, hot[k], o);
+      if ((threadIdx.x & 31) == 0) s[k][threadIdx.x >> 5][kGroup - 1] += hot[k];
     }
   }
   __syncthreads();

@@ -123,3 +123,39 @@ def test_statistics_of_few_and_many_samples(n):
     np.testing.assert_allclose(o[2:], t.std(1, ddof=1), rtol=1e-5)
     ref = (t.T.astype(np.float32) - o[:2]) / o[2:]
     np.testing.assert_allclose(Y.cpu().numpy(), ref, rtol=1e-5, atol=1e-5)
+
+
+# The standard deviation of n values moves by at most the largest error of one
+# of them: log10f's two last places of the largest value (equal values carry
+# equal errors; the temperature's float product has none).  The FP64 joins of
+# sum and sum of squares round at most a hundred times by 1.1e-16 of the mean
+# square (some 30 roundings in each of b, a and mu), the float results by 6e-8.
+@pytest.mark.parametrize("n", [300, 100_003])
+@pytest.mark.parametrize("spread", [0.0, 2e-6, 1e-5, 1e-4])
+def test_statistics_of_nearly_constant_features(n, spread):
+    rng = np.random.default_rng(n)
+    centre = np.linspace(-0.1, 0.1, I.NS)
+    centre[:5] = [0.0, 1e-3, 0.05, np.log10(0.866), np.log10(I.x_ss()[I.SIDX["X_aa"]])]
+    y = 10.0 ** (centre[:, None] + spread * rng.standard_normal((I.NS, n)))
+    T = 308.15 + 100.0 * spread * rng.standard_normal(n)
+    d = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    sc = torch.empty(CH.mlp_prep_scratch_bytes() // 8 + 1, dtype=torch.float64, device="cuda")
+    norm = torch.empty(64, device="cuda")
+
+    def check(T):
+        CH.chad_mlp_feature_norm(d(y), d(T), norm, sc)
+        f = np.vstack([np.log10(y.astype(np.float32).astype(np.float64)),
+                       (T.astype(np.float32) * np.float32(0.01)).astype(np.float64)])
+        nm = norm.cpu().numpy().astype(np.float64)
+        sd = np.maximum(f.std(1, ddof=1), 1e-6)
+        last = 2.0 * np.spacing(np.abs(f).max(1).astype(np.float32)).astype(np.float64)
+        last[29] = 0.0
+        assert np.all(np.abs(nm[:30] - f.mean(1)) <= last + 1e-6 * np.abs(f.mean(1)))
+        got = 1.0 / nm[32:62]
+        moved = last if spread > 0 else 0.0
+        var_tol = 100 * 1.1e-16 * (f ** 2).mean(1)
+        assert np.all(got ** 2 <= (sd * (1 + 1e-6) + moved) ** 2 + var_tol), got / sd
+        assert np.all(got ** 2 >= np.maximum(sd * (1 - 1e-6) - moved, 0.0) ** 2 - var_tol), got / sd
+
+    check(T)
+    check(T + 1.0e4)  # far above any digester's, still a number
