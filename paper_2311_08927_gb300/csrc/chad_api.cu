@@ -88,7 +88,8 @@ struct chad_ctx {
   double* d_atol = nullptr;
   DevCounters* d_cnt = nullptr;
   unsigned long long* d_queue = nullptr;
-  Migrant* d_mig = nullptr;    // particles on their way between threads (integrator tail)
+  Migrant* d_mig = nullptr;    // [mig_cap] particles on their way between threads (integrator tail)
+  int64_t mig_cap = 0;
   int* d_order = nullptr;      // [N] queue position -> particle, heaviest first
   int* d_order_cnt = nullptr;  // [2 * kOrderBuckets] bucket counts and cursors
   unsigned long long* d_misc = nullptr;  // [2]: load check flag, failed-particle count
@@ -319,7 +320,8 @@ chad_status chad_create(const chad_config* cfg, chad_ctx** out) {
   A(dalloc(&c->d_atol, NS));
   A(dalloc(&c->d_cnt, 1));
   A(dalloc(&c->d_queue, 1));
-  A(dalloc(&c->d_mig, (size_t)migrant_capacity(c->N, sms)));
+  c->mig_cap = migrant_capacity(c->N, sms);
+  A(dalloc(&c->d_mig, (size_t)c->mig_cap));
   A(dalloc(&c->d_order, c->N));
   A(dalloc(&c->d_order_cnt, 2 * kOrderBuckets));
   A(dalloc(&c->d_misc, 2));
@@ -864,6 +866,7 @@ static cudaError_t enqueue_interval(chad_ctx* c, double dt_days, int variant, cu
   a.h_learned = learned_now ? c->d_h_learned : nullptr;
   a.n_dig = c->n_dig;
   a.mig = c->d_mig;
+  a.mig_cap = c->mig_cap;
   cudaError_t e;
   if (learned_now) {
     const float* P = c->d_mlp;

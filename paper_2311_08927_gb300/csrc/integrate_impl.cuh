@@ -35,6 +35,7 @@
 
 #include <climits>
 #include <cstdint>
+#include <mutex>
 #include <type_traits>
 
 #include "adm1_device.cuh"
@@ -897,6 +898,50 @@ __global__ void __launch_bounds__(BS, MINB) integrate_kernel(StepArgs a) {
 
 }  // namespace integ
 
+// Resident blocks of a kernel instance on the current device.  The attributes
+// of the instance are set and its residency asked once per device, under a
+// lock: contexts of several devices and threads share the instance.
+struct ResidencyCache {
+  static constexpr int kDevices = 64;
+  std::mutex lock;
+  int64_t resident[kDevices] = {};
+};
+template <class K>
+cudaError_t resident_blocks(ResidencyCache& cache, K kernel, int threads, size_t smem,
+                            int64_t* resident) {
+  int dev = 0, sms = 0, per_sm = 0, smem_sm = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> hold(cache.lock);
+  const bool kept = dev >= 0 && dev < ResidencyCache::kDevices;
+  if (kept && cache.resident[dev] > 0) {
+    *resident = cache.resident[dev];
+    return cudaSuccess;
+  }
+  e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess && smem > 0)
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
+  if (e == cudaSuccess)
+    e = cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+  if (e != cudaSuccess) return e;
+  if (per_sm < 1) per_sm = 1;
+  // The unified L1 / shared array: the smallest shared carve-out that holds
+  // the resident blocks' tiles (none without a tile), so that the rest is L1
+  // for the spilled per-thread state whatever kernels ran before.  After the
+  // MLP training kernels (large shared tiles) the register shapes had less L1
+  // otherwise: 1M workload 46,279 -> 51,212 particle-days/s with the training
+  // in the same process.
+  const long long need = smem > 0 ? (long long)per_sm * ((long long)smem + 2048) : 0;
+  const int pct = smem_sm > 0 ? (int)((need * 100 + smem_sm - 1) / smem_sm) : 100;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, pct < 100 ? pct : 100);
+  if (e != cudaSuccess) return e;
+  *resident = (int64_t)sms * per_sm;
+  if (kept) cache.resident[dev] = *resident;
+  return cudaSuccess;
+}
+
 // Launch one kernel variant: persistent grid (resident blocks per SM x SMs,
 // capped by the particle count), queue head reset first.
 template <int FORM, int BS, int MINB, bool WS>
@@ -904,36 +949,12 @@ cudaError_t launch_variant(const StepArgs& a, cudaStream_t s) {
   using R = typename std::conditional<FORM == 1 || FORM == 2, float, double>::type;
   using LU = typename std::conditional<FORM == 3, spa::Lu, sp::Lu>::type;
   constexpr size_t smem = integ::wstore_smem_bytes<R, BS, WS, LU::nnz>();
-  static int per_sm = -1, sms = 0;
-  if (per_sm < 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (smem > 0) {
-      cudaError_t e = cudaFuncSetAttribute(integ::integrate_kernel<FORM, BS, MINB, WS>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-    }
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, integ::integrate_kernel<FORM, BS, MINB, WS>,
-                                                  BS, smem);
-    if (per_sm < 1) per_sm = 1;
-    // the smallest shared carve-out that holds the resident blocks' tiles
-    // (none without a tile): the rest of the unified array is L1 for the
-    // spilled per-thread state, whatever kernels ran before (a large-tile
-    // kernel otherwise leaves the shared share large)
-    int smem_sm = 0;
-    cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-    const long long need = smem > 0 ? (long long)per_sm * ((long long)smem + 2048) : 0;
-    const int pct = smem_sm > 0 ? (int)((need * 100 + smem_sm - 1) / smem_sm) : 100;
-    cudaError_t e = cudaFuncSetAttribute(integ::integrate_kernel<FORM, BS, MINB, WS>,
-                                         cudaFuncAttributePreferredSharedMemoryCarveout,
-                                         pct < 100 ? pct : 100);
-    if (e != cudaSuccess) return e;
-  }
-  int64_t blocks = (int64_t)sms * per_sm;
-  const int64_t need = (a.n + BS - 1) / BS;
-  if (need < blocks) blocks = need;
-  cudaError_t e = cudaMemsetAsync(a.queue, 0, sizeof(unsigned long long), s);
+  static ResidencyCache cache;
+  int64_t resident = 0;
+  cudaError_t e = resident_blocks(cache, integ::integrate_kernel<FORM, BS, MINB, WS>, BS, smem, &resident);
+  if (e != cudaSuccess) return e;
+  const int64_t blocks = grid_blocks(a.n, BS, resident, a.mig_cap);
+  e = cudaMemsetAsync(a.queue, 0, sizeof(unsigned long long), s);
   if (e != cudaSuccess) return e;
   integ::integrate_kernel<FORM, BS, MINB, WS><<<(unsigned)blocks, BS, smem, s>>>(a);
   return cudaGetLastError();

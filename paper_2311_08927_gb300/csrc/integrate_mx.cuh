@@ -625,38 +625,12 @@ __global__ void __launch_bounds__(BS, MINB) integrate_mx_kernel(StepArgs a) {
 template <int BS, int MINB, bool WS, bool IDX>
 cudaError_t launch_variant_mx_k(const StepArgs& a, cudaStream_t s) {
   constexpr size_t smem = integ::wstore_smem_bytes<float, BS, WS, spa::kNNZ>();
-  static int per_sm = -1, sms = 0;
-  if (per_sm < 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (smem > 0) {
-      cudaError_t e = cudaFuncSetAttribute(integ::integrate_mx_kernel<BS, MINB, WS, IDX>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-    }
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &per_sm, integ::integrate_mx_kernel<BS, MINB, WS, IDX>, BS, smem);
-    if (per_sm < 1) per_sm = 1;
-    // The unified L1 / shared array: the smallest shared carve-out that holds
-    // the resident blocks' tiles (none without a tile), so that the rest is
-    // L1 for the spilled per-thread state whatever kernels ran before.  After
-    // the MLP training kernels (large shared tiles) the register shapes had
-    // less L1 otherwise: 1M workload 46,279 -> 51,212 particle-days/s with
-    // the training in the same process.
-    int smem_sm = 0;
-    cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-    const long long need = smem > 0 ? (long long)per_sm * ((long long)smem + 2048) : 0;
-    const int pct = smem_sm > 0 ? (int)((need * 100 + smem_sm - 1) / smem_sm) : 100;
-    cudaError_t e = cudaFuncSetAttribute(integ::integrate_mx_kernel<BS, MINB, WS, IDX>,
-                                         cudaFuncAttributePreferredSharedMemoryCarveout,
-                                         pct < 100 ? pct : 100);
-    if (e != cudaSuccess) return e;
-  }
-  int64_t blocks = (int64_t)sms * per_sm;
-  const int64_t need = (a.n + BS - 1) / BS;
-  if (need < blocks) blocks = need;
-  cudaError_t e = cudaMemsetAsync(a.queue, 0, sizeof(unsigned long long), s);
+  static ResidencyCache cache;
+  int64_t resident = 0;
+  cudaError_t e = resident_blocks(cache, integ::integrate_mx_kernel<BS, MINB, WS, IDX>, BS, smem, &resident);
+  if (e != cudaSuccess) return e;
+  const int64_t blocks = grid_blocks(a.n, BS, resident, a.mig_cap);
+  e = cudaMemsetAsync(a.queue, 0, sizeof(unsigned long long), s);
   if (e != cudaSuccess) return e;
   integ::integrate_mx_kernel<BS, MINB, WS, IDX><<<(unsigned)blocks, BS, smem, s>>>(a);
   return cudaGetLastError();

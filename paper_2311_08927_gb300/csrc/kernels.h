@@ -19,7 +19,7 @@ struct DevCounters {
 };
 
 // A particle between two attempts, as it moves to another thread of its block
-// (see compact() in integrate_impl.cuh); its states travel through y.
+// (see rank_in_block in integrate_impl.cuh); its states travel through y.
 struct Migrant {
   long long p;
   double SH, SH2, h, t;
@@ -52,7 +52,8 @@ struct StepArgs {
   const double* SH_learned;   // learned guesses for particles without history (or null)
   const double* h_learned;
   int n_dig;                  // digesters of the context
-  Migrant* mig;               // [migrant_capacity(n, SMs)] scratch
+  Migrant* mig;               // [mig_cap] scratch
+  int64_t mig_cap;            // migrant_capacity(n, SMs) of the context's device
 };
 
 struct AdvectArgs {
@@ -119,6 +120,14 @@ constexpr int default_variant(int form, int64_t n, int sms) {
 // Entries of StepArgs::mig: one per resident thread of the persistent grid.
 constexpr int64_t migrant_capacity(int64_t n, int sms) {
   return n + 256 < (int64_t)sms * 2048 ? n + 256 : (int64_t)sms * 2048;
+}
+// Blocks of the persistent grid: one per `threads` particles, at most the
+// resident ones, and never more than the scratch has entries for, whatever
+// device the residency was asked of.
+constexpr int64_t grid_blocks(int64_t n, int threads, int64_t resident, int64_t mig_cap) {
+  const int64_t need = (n + threads - 1) / threads, room = mig_cap / threads;
+  const int64_t most = resident < room ? resident : room;
+  return need < most ? need : most;
 }
 cudaError_t launch_integrate(const StepArgs& a, int precision, int variant, cudaStream_t s);
 cudaError_t launch_advect(const AdvectArgs& a, cudaStream_t s);
