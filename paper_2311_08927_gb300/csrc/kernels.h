@@ -108,14 +108,23 @@ constexpr KernelVariant kernel_variant(int form, int v) {
 // spread them over the SMs, so that a warp has its sub-partition's FP64 pipe
 // (one warp instruction per 64 cycles) to itself: 1,000 particles FP64 with
 // S_h2 algebraic 2.92 ms with 128-thread blocks, 2.70 with 64, 2.68 with 32;
-// 12,000 particles FP64 9.72 ms, 9.37, 9.58.  From 128 particles per SM on,
-// large blocks, whose warps share the fetched code: 30,000 particles FP64
-// 11.4 ms with 128 threads, 13.0 with 64.  There form 4 takes one block of
-// eight warps per SM with W_d in shared memory: 64 digesters with 400,000
-// particles 115.9 ms (128 threads, W_d in registers) against 83.1, 1M
-// particles with slugs 34.0 against 27.1.
+// 12,000 particles FP64 9.72 ms, 9.37, 9.58.  (Form 4, first / third interval
+// of a population with slugs: 2,500 particles 5.65 / 3.13 ms with 128 threads,
+// 5.54 / 3.03 with 64, 5.43 / 2.96 with 32; 12,000 particles 6.28 / 3.18,
+// 6.29 / 3.07, 6.42 / 3.05.)  From 128 particles per SM on, large blocks, whose
+// warps share the fetched code: 30,000 particles FP64 11.4 ms with 128
+// threads, 13.0 with 64; 26,000 particles form 4 7.28 / 3.58 and 9.32 / 3.99.
+// Form 4 goes on to one block of eight warps per SM with W_d in shared memory
+// where nearly all SMs get one: 64 digesters with 400,000 particles 115.9 ms
+// (128 threads, W_d in registers) against 83.1, 1M particles with slugs 34.0
+// against 27.1, 38,912 particles 9.21 / 4.72 against 8.74 / 4.69; with fewer
+// particles SMs stay empty: 36,000 particles 8.81 / 4.66 against 8.77 / 4.50,
+// 33,000 7.96 / 4.22 against 8.28 / 4.50, 22,000 7.02 / 3.30 against
+// 8.64 / 4.37.  The line at 232 per SM (35,264) lies between 33,000 and 36,000.
 constexpr int default_variant(int form, int64_t n, int sms) {
-  return n <= (int64_t)64 * sms ? 5 : n <= (int64_t)128 * sms ? 3 : form == 4 ? 6 : 0;
+  if (n <= (int64_t)64 * sms) return 5;
+  if (n <= (int64_t)128 * sms) return 3;
+  return form == 4 && n > (int64_t)232 * sms ? 6 : 0;
 }
 // Entries of StepArgs::mig: one per resident thread of the persistent grid.
 constexpr int64_t migrant_capacity(int64_t n, int sms) {

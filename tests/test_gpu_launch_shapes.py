@@ -45,6 +45,16 @@ def test_default_shape_equals_an_explicit_one(sms, kw, tol, per_sm, extra):
     assert np.array_equal(a["status"], b["status"])
 
 
+@pytest.mark.parametrize("extra", [0, 1])
+def test_mixed_default_shape_around_the_line_of_the_large_blocks(sms, extra):
+    kw = dict(precision=CH.PREC_MIXED, h2_algebraic=True)
+    pop = I.config_population(3, n=232 * sms + extra)
+    a, b = _run(pop, None, **kw), _run(pop, 5, **kw)
+    floor = 1e-12 * np.abs(b["y"]).max(axis=1, keepdims=True) + 1e-300
+    assert (np.abs(a["y"] - b["y"]) / np.maximum(np.abs(b["y"]), floor)).max() <= 1e-6
+    assert np.array_equal(a["status"], b["status"])
+
+
 def _adaptive(pop, variant, **kw):
     sim = CH.Simulator(pop, **kw)
     CH.chad_set_kernel_variant(sim.ctx, variant)
