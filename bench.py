@@ -167,7 +167,7 @@ def alu_roofline(f64, f32, launch_ms, peak64, peak32):
 def kernel_sources_hash():
     import hashlib
     h = hashlib.sha256()
-    for f in ("adm1_device.cuh", "integrate_impl.cuh", "integrate_mx.cuh", "dfloat.cuh", "rank1.cuh",
+    for f in ("adm1_device.cuh", "error_norm.cuh", "integrate_impl.cuh", "integrate_mx.cuh", "dfloat.cuh", "rank1.cuh",
               "sparse_lu_gen.cuh", "sparse_lu_h2a_gen.cuh", "model.h", "kernels.h"):
         with open(os.path.join(ROOT, "paper_2311_08927_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())

@@ -88,10 +88,14 @@ template <class R>
 CHAD_HD R rcp(R d) {
   return R(1) / d;
 }
-__device__ __forceinline__ float rcp_approx(float d) {
+CHAD_HD float rcp_approx(float d) {
+#ifdef __CUDA_ARCH__
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
   return r;
+#else
+  return 1.0f / d;
+#endif
 }
 #ifdef __CUDA_ARCH__
 template <>

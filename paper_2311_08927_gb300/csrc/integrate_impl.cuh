@@ -39,6 +39,7 @@
 #include <type_traits>
 
 #include "adm1_device.cuh"
+#include "error_norm.cuh"
 #include "kernels.h"
 #include "rank1.cuh"
 #include "sparse_lu_gen.cuh"
@@ -371,14 +372,6 @@ struct H2Split {
     return s < spa::kNNZ ? w[s] : (s < spa::kNNZ + NS ? row[s - spa::kNNZ] : col[s - spa::kNNZ - NS]);
   }
 };
-
-// |d| as a float from its high word: truncated to 20 significand bits, below
-// the normal float range zero, above it (and for infinities and NaN) infinite.
-__device__ __forceinline__ float magf(double d) {
-  int m = (__double2hiint(d) & 0x7fffffff) - 0x38000000;
-  m = min(max(m, 0), 0x0ff00000);
-  return __uint_as_float((unsigned)m << 3);
-}
 
 // norm^(-1/3) of the step controller
 __device__ __forceinline__ float inv_cbrt(float x) { return rcbrtf(x); }
@@ -765,34 +758,11 @@ __global__ void __launch_bounds__(BS, MINB) integrate_kernel(StepArgs a) {
       // no error norm (its finiteness: in the last stage)
     } else if (piv_ok || fixed) {
       // scaled error norm max_i |h/6 (k1 - 2 k2 + k3)_i| / (atol_i + rtol
-      // max(|y_i|, |y1_i|)).  FP64 forms: all of it in FP64, as the oracle.
+      // max(|y_i|, |y1_i|)).  FP64 forms: in FP64, as the oracle (error_norm.cuh).
       // Mixed forms: the combination, which cancels, in FP64, everything
       // after it in FP32 (the accept test needs a few digits only).
       if constexpr (!MIXED) {
-        // The species with the largest ratio is found in FP32 (truncated
-        // high words, a few 1e-6 relative), its error and magnitude kept in
-        // FP64 and the norm formed from them: a near tie can pick a ratio
-        // 4e-6 below the largest.  Comparing 29 ratios in FP64 took five
-        // slots of the FP64 pipe per species.  Not finite: an infinite norm.
-        double en = 0.0, ym = 0.0, at = 1.0;
-        float best = 0.0f;
-        const float rtol = cvt<float>(a.rtol);
-#pragma unroll
-        for (int i = 0; i < NS; ++i) {
-          const double e = fma(-2.0, k2[i], k1[i]) + xs[i];
-          const double yi = mag64(y[i]) > mag64(y1[i]) ? y[i] : y1[i];
-          const float ef = magf(e), yf = magf(yi);
-          const float r = ef * rcp_approx(fmaf(rtol, yf, magf(a.atol[i])));
-          const bool inf = ef == INFINITY || yf == INFINITY;
-          if (inf ? best < INFINITY : r > best) {
-            best = inf ? INFINITY : r;
-            en = e;
-            ym = yi;
-            at = a.atol[i];
-          }
-        }
-        const double sn = fma(a.rtol, fabs(ym), at);
-        norm = best == INFINITY ? NR(INFINITY) : fabs(en) * rcp<double>(sn) * (hh * (1.0 / 6.0));
+        norm = error_ratio(y, y1, k1, k2, xs, a.rtol, a.atol) * (hh * (1.0 / 6.0));
       } else {
         float nf = 0.0f;
         const float rtol = cvt<float>(a.rtol);
