@@ -126,7 +126,7 @@ class ClockSampler:
 
 
 # --------------------------------------------------------------------------- algorithmic work
-def work_per_launch(CH, precision, stats, steps, h2=False):
+def work_per_launch(CH, precision, stats, steps, h2=False, fixed=False):
     """Algorithmic FP64 / FP32 operations of one integrator launch.
 
     Counts come from the kernel source (chad_flop_counts: the templated
@@ -137,17 +137,18 @@ def work_per_launch(CH, precision, stats, steps, h2=False):
     iteration of Eq. 7 one charge-balance evaluation plus the update; per
     attempt three moves of the acid-base reciprocals to the converged root.
     The mixed form with S_h2 algebraic counts its two-float arithmetic at its
-    FP32 cost and each FP32 Eq. 8 Newton iteration."""
+    FP32 cost and each FP32 Eq. 8 Newton iteration.  Fixed substeps do
+    without the error estimate and what it alone needs."""
     nf = CH.newton_flops()
     fin = CH.flop_counts()["sh_final"]
     attempts = stats["accepted_steps"] + stats["rejected_steps"]
     if h2 and precision == CH.PREC_MIXED:
-        af = CH.attempt_flops_h2_mixed()
+        af = CH.attempt_flops_h2_mixed(fixed)
         f32 = attempts * af["fp32"] + stats["h2_newton_iters"] * af["fp32_per_h2_iter"]
     else:
-        af = CH.attempt_flops(precision, h2)
+        af = CH.attempt_flops(precision, h2, fixed)
         f32 = attempts * af["fp32"]
-    f64 = attempts * (af["fp64"] + 3 * fin) + stats["newton_iters"] * nf
+    f64 = attempts * (af["fp64"] - af.get("fp64_zero", 0) + 3 * fin) + stats["newton_iters"] * nf
     if "fp64_per_h2_iter" in af:
         f64 += stats["h2_newton_iters"] * af["fp64_per_h2_iter"]
     return f64 / steps, f32 / steps, af
@@ -677,7 +678,7 @@ def run_fig7(args, ws, rank, local):
     ms = e0.elapsed_time(e1)
     st = sim.read()["stats"]
     sim.close()
-    f64, _, af = work_per_launch(CH, CH.PREC_FP64, st, k)
+    f64, _, af = work_per_launch(CH, CH.PREC_FP64, st, k, fixed=True)
     achieved = f64 / (ms / k * 1e-3) / 1e12
     days = FIG7_DT_S / 86400.0
     res = {"metric": "particle-days simulated per second (paper-literal stepping)",

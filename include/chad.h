@@ -488,9 +488,9 @@ chad_status chad_probe_alu_peak(int fp64, double* tflops);
    refinement update of one mixed solve (with its rank-1 term), out[9]
    Sherman-Morrison set-up of one attempt (q = (I - g J_d)^-1 g u and its
    denominator, besides the sparse solve), out[10] Sherman-Morrison update
-   of one solve, out[11] move of the Eq. 7 reciprocals and slope to a
-   converged root, out[12] scaling of the rate partials by -g (the FP64
-   form's formation of I - g J_d, with one add per diagonal).  n >= 13.
+   of one solve, out[11] once per Eq. 7 solve: its products, the third-order
+   step and the move of the reciprocals and slope to the root, out[12] 0 (the
+   scaling of the rate partials by -g is part of out[1]).  n >= 13.
    With n >= 18 also the mixed form with S_h2 algebraic: out[13] J x from
    the FP32 rate partials in two-float arithmetic (in FP32 flops), out[14]
    the Eq. 8 balance coefficients, out[15] one Eq. 8 Newton iteration,
@@ -499,7 +499,12 @@ chad_status chad_probe_alu_peak(int fp64, double* tflops);
    work (evaluation points, S_H guesses); with n >= 19 out[18] the rates
    with their partials alone; with n >= 22 out[19] W formation, out[20]
    LU and out[21] one solve of the LU without S_h2's row and column, which
-   the forms with S_h2 algebraic factor. */
+   the forms with S_h2 algebraic factor; with n >= 28 out[22] the entries of
+   dS_h2/dy and out[23] those of the second Sherman-Morrison vector (products
+   with the others are left out), out[24] the rate factors that Eq. 8 and the
+   rates share (part of out[0], [1] and [18]), out[25] the share of one stage
+   in out[16], out[26] and out[27] the shares in out[16] and out[7] of the
+   third right-hand side and the error norm, which fixed steps do without. */
 chad_status chad_flop_counts(int64_t* out, int n);
 
 /* The integrator's device arithmetic helpers applied to x [n] (host

@@ -295,7 +295,8 @@ def chad_mlp_adam(params, grad, m, v, t, lr, beta1=0.9, beta2=0.999, eps=1e-8, s
 FLOP_KEYS = ["rates_f", "rates_fj", "charge_E", "form_w", "factor", "solve", "jx", "stage",
              "refine", "sm_setup", "sm_update", "sh_final", "scale_j", "jx_twofloat",
              "h2_coeffs", "h2_iter", "mx_fp32_extra", "mx_fp64_extra", "rates_partials",
-             "form_w_h2a", "factor_h2a", "solve_h2a"]
+             "form_w_h2a", "factor_h2a", "solve_h2a", "h2_reads", "h2_moves", "factors",
+             "mx_stage", "mx_third", "third"]
 
 
 def flop_counts() -> dict:
@@ -306,7 +307,7 @@ def flop_counts() -> dict:
     return dict(zip(FLOP_KEYS, (int(x) for x in out)))
 
 
-def attempt_flops_h2_mixed() -> dict:
+def attempt_flops_h2_mixed(fixed_substeps: bool = False) -> dict:
     """FP64 and FP32 operations of one step attempt of the mixed form with
     S_h2 algebraic (kernel form 4), without the Newton iterations of Eq. 7
     (FP64) and Eq. 8 (FP32), which are counted per iteration: FP32 rates with
@@ -316,16 +317,21 @@ def attempt_flops_h2_mixed() -> dict:
     partials recomputed for each of the three refinement residuals and
     their two-float J x, and the two-float stage arithmetic;
     FP64 for the evaluation points and the S_H guesses.  The LU is the one
-    without S_h2's row and column (spa)."""
+    without S_h2's row and column (spa).  A fixed substep has no error
+    estimate and leaves the third stage after its two roots."""
     f = flop_counts()
     f32 = (f["rates_fj"] + 2 * f["rates_f"] + f["form_w_h2a"] + f["factor_h2a"] +
            8 * f["solve_h2a"] +
            f["sm_setup"] + 7 * f["sm_update"] + 3 * f["h2_coeffs"] + 3 * f["jx_twofloat"] +
            3 * f["rates_partials"] + f["mx_fp32_extra"])
+    if fixed_substeps:
+        f32 -= (f["rates_f"] - f["factors"] + 2 * f["solve_h2a"] + 2 * f["sm_update"] +
+                f["jx_twofloat"] + f["rates_partials"] + f["mx_stage"] + f["mx_third"])
     return {"fp64": f["mx_fp64_extra"], "fp32": f32, "fp32_per_h2_iter": f["h2_iter"]}
 
 
-def attempt_flops(precision: int, h2_algebraic: bool = False) -> dict:
+def attempt_flops(precision: int, h2_algebraic: bool = False,
+                  fixed_substeps: bool = False) -> dict:
     """FP64 and FP32 operations of one W-method step attempt, without the
     Eq. 7 Newton iterations (counted separately per iteration).  The linear
     algebra is the Sherman-Morrison form: one LU of I - g J_d, one solve for
@@ -336,7 +342,10 @@ def attempt_flops(precision: int, h2_algebraic: bool = False) -> dict:
     a fifth solve for the second Sherman-Morrison vector p2 and its update
     of each stage, the Eq. 8 coefficients at the three evaluation points and
     the S_h2 tangent guesses (its Newton iterations counted per iteration,
-    h2_iter)."""
+    h2_iter); "fp64_zero" is what "fp64" counts there for products with
+    entries of dS_h2/dy and p2 that are always zero, which the kernel leaves
+    out.  The FP64 forms' fixed substeps have no error estimate and leave out
+    the third stage's right-hand side, solve and updates."""
     f = flop_counts()
     if precision == PREC_FP64 and h2_algebraic:
         # W_d as in the FP64 form over the 28 states of spa; p2: solve, first
@@ -346,11 +355,18 @@ def attempt_flops(precision: int, h2_algebraic: bool = False) -> dict:
         f64 = (f["rates_fj"] + 2 * f["rates_f"] + f["scale_j"] + (NS - 1) + f["factor_h2a"] +
                5 * f["solve_h2a"] + f["sm_setup"] + 4 * f["sm_update"] + f["stage"] +
                3 * f["h2_coeffs"] + 59 + 54 + 3 * 117 + 2 * 58)
-        return {"fp64": f64, "fp32": 0, "fp64_per_h2_iter": f["h2_iter"]}
+        dots, moves = 2 * (NS - f["h2_reads"]), 2 * (NS - f["h2_moves"])
+        zero = 3 * dots + 3 * (dots + moves)
+        if fixed_substeps:
+            f64 -= f["solve_h2a"] + f["sm_update"] + 117 + f["third"]
+            zero -= dots + moves
+        return {"fp64": f64, "fp32": 0, "fp64_zero": zero, "fp64_per_h2_iter": f["h2_iter"]}
     if precision == PREC_FP64:
         # W_d: the rate partials scaled by -g before the scatter, plus the diagonal ones
         f64 = (f["rates_fj"] + 2 * f["rates_f"] + f["scale_j"] + NS + f["factor"] +
                4 * f["solve"] + f["sm_setup"] + 3 * f["sm_update"] + f["stage"])
+        if fixed_substeps:
+            f64 -= f["solve"] + f["sm_update"] + f["third"]
         return {"fp64": f64, "fp32": 0}
     f32_rates = precision == PREC_MIXED_F32RATES
     f64 = 3 * (f["jx"] + f["refine"]) + f["stage"] + (0 if f32_rates else 3 * f["rates_f"])

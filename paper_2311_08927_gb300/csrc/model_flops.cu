@@ -93,6 +93,13 @@ using namespace chad;
 // out[16] FP32 work of one attempt besides rates, LU, solves, J x and Eq. 8
 // out[17] FP64 work of one attempt besides the Eq. 7 Newton iterations
 // With n >= 19: out[18] the rates with their partials alone (rates<., true>).
+// With n >= 28:
+// out[22] entries of dS_h2/dy (h2_reads)
+// out[23] entries that the second Sherman-Morrison vector moves (h2_moves)
+// out[24] the rate factors shared by Eq. 8 and the rates (part of out[0], [1], [18])
+// out[25] out[16]'s share of one stage's solve and refinement
+// out[26] out[16]'s share of the third right-hand side and the error norm
+// out[27] out[7]'s share of the same
 extern "C" chad_status chad_flop_counts(int64_t* out, int n) {
   if (!out || n < 13) return CHAD_E_INVALID;
   DigConst c;
@@ -177,6 +184,11 @@ extern "C" chad_status chad_flop_counts(int64_t* out, int n) {
   out[7] = (int64_t)NS * 18;
   // s = v^T x (15), b - x + g jx (3/elt), x += dx (1/elt)
   out[8] = 15 + (int64_t)NS * 4;
+  int64_t nr = 0, nm = 0;
+  for (int i = 0; i < NS; ++i) {
+    nr += h2_reads(i);
+    nm += h2_moves(i);
+  }
   if (n >= 18) {
     {
       DFc x[NS], jx[NS];
@@ -200,17 +212,22 @@ extern "C" chad_status chad_flop_counts(int64_t* out, int n) {
     // FP32 flops of one form-4 attempt outside the counted blocks, from the
     // kernel source (two-float operations at their FP32 cost: TwoSum 6,
     // TwoProd 3, a sum with a float 10, a sum 11, a product 10, a product
-    // with a float 8):
+    // with a float 8); nr entries of dS_h2/dy, nm of p2:
     //   S_h2 surgery of J_d: zh (29 + 3 x 8), p2 (29), its reciprocal (1)   83
-    //   q scaling (29), second-level dot and denominator (58 + 3)           90
-    //   per stage (x3): two wsolve level-2 updates (2 x (58 + 1 + 58)),
-    //     x'_h2 = zh^T x (28 x 13), v^T x (8 x 13), residual b - x + g J x
-    //     (29 x 32), x = x0 + dx (29)                          234 + 364 + 104 + 928 + 29
+    //   q scaling (29), second-level dot and denominator (2 nr + 3)
+    //   per stage (x3): two wsolve level-2 updates (2 x (2 nr + 1 + 2 nm)),
+    //     x'_h2 = zh^T x (nr x 13), v^T x (8 x 13), residual b - x + g J x
+    //     (29 x 32), x = x0 + dx (29)
     //   k2 = x + k1 (29); right-hand sides: stage 1 (29 x 17 with
     //     C = e32 F1 + 2 F0), stage 2 (29 x 40), stage-1 float point (29 x 2)
     //   error norm: k1 - 2 k2 + k3 exact (17), hi + lo (1), scale (4)   29 x 22
-    out[16] = 83 + 90 + 3 * (234 + 28 * 13 + 8 * 13 + (int64_t)NS * 32 + NS) + NS +
-              (int64_t)NS * (17 + 40 + 2) + (int64_t)NS * 22;
+    const int64_t stage = 2 * (2 * nr + 1 + 2 * nm) + nr * 13 + 8 * 13 + (int64_t)NS * 32 + NS;
+    const int64_t third = (int64_t)NS * (40 + 22);
+    out[16] = 83 + NS + 2 * nr + 3 + 3 * stage + NS + (int64_t)NS * (17 + 2) + third;
+    if (n >= 28) {
+      out[25] = stage;
+      out[26] = third;
+    }
     // FP64 flops of one form-4 attempt besides the Eq. 7 iterations (and the
     // three root moves, counted with them): evaluation points y + (h/2) k1 in
     // the 8 states of Eq. 7 and y + h k2 in all 29 (one FMA each), the two
@@ -241,6 +258,14 @@ extern "C" chad_status chad_flop_counts(int64_t* out, int n) {
     g_ops = 0;
     spa::solve<Fc>(wa, ba);
     out[21] = g_ops;
+  }
+  if (n >= 28) {
+    out[22] = nr;
+    out[23] = nm;
+    g_ops = 0;
+    factors<Fc>(c, q, y, ab, k);
+    out[24] = g_ops;
+    out[27] = (int64_t)NS * (5 + 4 + 2 + 1);
   }
   return CHAD_OK;
 }

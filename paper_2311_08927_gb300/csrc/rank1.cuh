@@ -18,6 +18,23 @@
 #include "sparse_lu_gen.cuh"
 
 namespace chad {
+
+// the eight states that enter Eq. 7
+__host__ __device__ constexpr bool in_eq7(int i) {
+  return i == iS_va || i == iS_bu || i == iS_pro || i == iS_ac || i == iS_IC || i == iS_IN ||
+         i == iS_cat || i == iS_an;
+}
+// S_h2 algebraic: the states that dS_h2/dy reaches (the S_h2 row of the
+// Jacobian and, through S_H, the states of Eq. 7), and those that the second
+// Sherman-Morrison vector p2 reaches (not the two ions, which only dilute,
+// nor S_h2 itself).  Products with the other entries are left out.
+__host__ __device__ constexpr bool h2_reads(int j) {
+  return j != iS_h2 && (sp::slot(iS_h2, j) >= 0 || in_eq7(j));
+}
+__host__ __device__ constexpr bool h2_moves(int i) {
+  return i != iS_h2 && i != iS_cat && i != iS_an;
+}
+
 namespace rank1 {
 
 // v^T x over the eight states of Eq. 7 (v[k] belongs to state hc[k]).
