@@ -79,10 +79,15 @@ __device__ __forceinline__ float cvt<float, double>(double d) {
 //     then one polynomial correction r0 (1 + e + e^2) of the Newton-Raphson
 //     family for the reciprocal, whose relative error is O(e^3) (below
 //     1e-18): three FMAs on the FP64 pipe.  |d| below 2^-1022 gives a
-//     signed infinity, |d| from 2^1022 on a signed zero, NaN stays NaN.
+//     signed infinity, |d| from 2^1022 on a signed zero.  A NaN stays one as
+//     long as its high word says so, which every operation's result does (a
+//     payload in the low word alone would read as an infinity).
 //   FP32: the approximate reciprocal and one Newton-Raphson step with the
-//     residual from an FMA (rounded to nearest but for near-ties); d = 0,
-//     infinite or NaN keeps the approximation, which is exact there.
+//     residual from an FMA: correctly rounded for all normal d with a normal
+//     reciprocal (all 2^32 arguments tested).  d = 0, infinite or NaN keeps
+//     the approximation, which is exact there, and so do subnormal d (signed
+//     infinity) and |d| above 2^126 (signed zero): the kernels' arguments are
+//     sums with a half-saturation or scale constant, pivots near 1 and slopes.
 // Elsewhere (host, counting types): the plain division.
 template <class R>
 CHAD_HD R rcp(R d) {
