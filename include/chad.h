@@ -245,8 +245,10 @@ chad_status chad_debug_bounds(int32_t* enabled, uint32_t* status, int reset);
    noise (0 after chad_create, +1 per interval), so a run restored from a
    checkpoint continues bit for bit when it is put back: save y, pos, S_H, h
    (chad_read_states), T and this index; restore with chad_load_particles
-   (with S_H and h) for every digester, then chad_set_interval.  Both wait
-   for the context's stream. */
+   (with S_H and h) for every digester, then chad_set_interval.  That holds
+   for a context of the same configuration and particle count (or one with
+   the same kernel variant set, see chad_set_kernel_variant).  Both wait for
+   the context's stream. */
 chad_status chad_get_interval(chad_ctx* ctx, uint64_t* interval);
 chad_status chad_set_interval(chad_ctx* ctx, uint64_t interval);
 
@@ -322,7 +324,14 @@ chad_status chad_autotune(chad_ctx* ctx, double dt_coupling_s, int32_t* chosen, 
 /* Use kernel variant v (0 <= v < CHAD_NUM_VARIANTS) for this context's
    kernel form from the next chad_step on, in place of the default (chosen by
    the particle count) or the autotuner's choice: a fixed launch shape, e.g.
-   for reproducible timing.  Results do not depend on the variant. */
+   for reproducible timing.  With the same variant, configuration and inputs
+   a run repeats bit for bit.  Variants are different compilations of the same
+   arithmetic: fixed steps agree to round-off; adaptive ones may be accepted a
+   little differently (FP64 states agree to 1e-10 or better, the mixed forms'
+   within the tolerance of the steps).  Since the default follows the particle
+   count, shards of a population that have to match it bit for bit set one
+   variant for all (and, with CHAD_PREC_MIXED and h2_algebraic, are not split
+   between contexts of one digester and contexts of several). */
 chad_status chad_set_kernel_variant(chad_ctx* ctx, int variant);
 
 /* The launch shape of kernel variant v (0 <= v < CHAD_NUM_VARIANTS) for a

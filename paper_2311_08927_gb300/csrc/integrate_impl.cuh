@@ -84,12 +84,13 @@ __device__ __forceinline__ int64_t queue_pop(unsigned long long* q) {
 // move to its first threads, so that half the warps go idle and the others
 // have the sub-partitions' FP64 pipes (one warp instruction per 64 cycles,
 // whatever its active lanes) to themselves.  With one to three particles per
-// thread the tail is a third of an interval: 60,000 particles FP64 17.2 ->
-// 15.7 ms, 100,000 in the cylinder 45.2 -> 43.1, 5,000 mixed (64-thread
-// blocks) 1.64 -> 1.43.  The mixed form's 256-thread blocks, which serve many
-// particles per thread, gain nothing and lose 6 % to the added code: they do
-// without.  rank_in_block gives the place (valid where `act`) and the number
-// of particles; every thread of the block calls it.
+// thread the tail is a third of an interval: 60,000 particles FP64 17.2 ms
+// without the moves, 15.7 with them; 100,000 in the cylinder 45.2 and 43.1.
+// A 32-thread block, the default for few particles, has no other warp to move
+// to; the mixed form's 256-thread blocks, which serve many particles per
+// thread, gain nothing and lose 6 % to the added code: they do without.
+// rank_in_block gives the place (valid where `act`) and the number of
+// particles; every thread of the block calls it.
 template <int BS>
 __device__ __forceinline__ int rank_in_block(bool act, int* warp_count, int& total) {
   const unsigned m = __ballot_sync(0xffffffffu, act);
@@ -592,7 +593,8 @@ __global__ void __launch_bounds__(BS, MINB) integrate_kernel(StepArgs a) {
                fabs(delta2) >= kPivTau * fmax(1.0, fabs(s2));
     }
     }
-    // error norm and controller: FP64 in the FP64 forms, FP32 in the mixed ones
+    // error norm and controller: FP64 in the FP64 forms (its species found in
+    // FP32 where that is sure), FP32 in the mixed ones
     using NR = typename std::conditional<MIXED, float, double>::type;
     NR norm = NR(INFINITY);
     if (!MIXED && act && !piv_ok) cnt.pivot++;

@@ -1,8 +1,8 @@
 """Particles that move between the threads of a block at the end of an interval
 (the 128-thread shape) against the 32-thread shape, which never moves any:
 populations of many digesters (a moved particle takes its own digester's
-constants along) and cold starts from learned guesses (the count of guesses
-done anew travels with the particle)."""
+constants along), cold starts from learned guesses (the count of guesses done
+anew travels with the particle) and shards of a population."""
 import numpy as np
 import pytest
 
@@ -66,3 +66,17 @@ def test_moved_particles_keep_their_learned_start(kw, tol):
     # the guesses, and which of them are done anew, are the same in both runs
     _same(a, b, tol, ("mlp_redo",))
     assert 0 < a["stats"]["accepted_steps"]
+
+
+@pytest.mark.parametrize("kw,tol", FORMS)
+def test_shards_with_one_variant_match_the_whole_bit_for_bit(kw, tol):
+    """A default launch shape follows the particle count; with the variant set
+    a particle's run does not depend on the others, whichever thread ends it."""
+    pop = I.config_population(3, n=N)
+    whole = _run(pop, 0, **kw)
+    for a, b in ((0, 700), (700, N)):
+        part = I.Population([I.Digester(n=b - a)], np.ascontiguousarray(pop.y[:, a:b]), pop.T[a:b],
+                            np.ascontiguousarray(pop.pos[:, a:b]), False, "shard")
+        out = _run(part, 0, **kw)
+        for k in ("y", "S_H", "h", "status"):
+            assert np.array_equal(out[k], whole[k][..., a:b]), k
